@@ -277,6 +277,8 @@ std::vector<uint64_t> workspace_signature(const tigre_geometry* g);
 // single-volume operators' bit for bit.
 tigre_status forward_batch_impl(tigre_geometry* g, const void* vols, void* projs, int batch,
                                  tigre_dtype dt, void* const quad[2], cudaStream_t st);
+// Which of the two quad workspaces a batched projection reads.
+void batch_quad_layouts(const tigre_geometry* g, bool need[2]);
 size_t backward_batch_workspace_bytes(const tigre_geometry* g, tigre_dtype dt);
 tigre_status backward_batch_impl(tigre_geometry* g, const void* projs, void* vols, int batch,
                                  tigre_dtype dt, tigre_bp_weight w, void* ws, cudaStream_t st);

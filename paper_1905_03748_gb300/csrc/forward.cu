@@ -27,6 +27,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "forward_cols.cuh"
 #include "quad.cuh"
 #include "ray.cuh"
 
@@ -204,8 +205,8 @@ __device__ __forceinline__ float tri_sample(const TV* __restrict__ vol, const Ra
     const float v010 = ld(b + PF), v110 = ld(b + PF + 1);
     const float v001 = ld(b + PFM), v101 = ld(b + PFM + 1);
     const float v011 = ld(b + PFM + PF), v111 = ld(b + PFM + PF + 1);
-    const float c0 = bilinear_value(bilinear_coefficients(v000, v100, v010, v110), af, am);
-    const float c1 = bilinear_value(bilinear_coefficients(v001, v101, v011, v111), af, am);
+    const float c0 = bilinear_fm(R.layout, v000, v100, v010, v110, af, am);
+    const float c1 = bilinear_fm(R.layout, v001, v101, v011, v111, af, am);
     return fmaf(as, c1 - c0, c0);
 }
 
@@ -341,7 +342,8 @@ __global__ void __launch_bounds__(256) quad_from_vol_kernel(const T* __restrict_
         const T a = tile[i][threadIdx.x], b = tile[i][threadIdx.x + 1];
         const T c = tile[i + 1][threadIdx.x], d = tile[i + 1][threadIdx.x + 1];
         typename QuadOf<T>::type* o = out + ((int64_t)s * PM + m) * PF + f;
-        *o = bilinear_coefficients(to_f32<T>(a), to_f32<T>(b), to_f32<T>(c), to_f32<T>(d));
+        *o = layout ? bilinear_coefficients(to_f32<T>(a), to_f32<T>(c), to_f32<T>(b), to_f32<T>(d))
+                    : bilinear_coefficients(to_f32<T>(a), to_f32<T>(b), to_f32<T>(c), to_f32<T>(d));
     }
 }
 
@@ -367,7 +369,7 @@ __host__ __device__ __forceinline__ uint32_t quad_index_bias(int PF, int PFM, in
 
 // Trilinear sample kf of a ray from the quad volume qv; ym = x0[1] + kf d[1]
 // (the march's depth coordinate, which the caller has already formed).
-template <typename TV>
+template <typename TV, bool LAYOUT1>
 __device__ __forceinline__ float tri_sample_quad(const typename QuadOf<TV>::type* __restrict__ qv,
                                                  const Ray& R, float kf, float ym, int PF, int PFM,
                                                  uint32_t bias)
@@ -379,8 +381,9 @@ __device__ __forceinline__ float tri_sample_quad(const typename QuadOf<TV>::type
     split_bits(fmaf(kf, R.d[2], R.x0[2]), b_s, as);
     const uint32_t e = b_s * (uint32_t)PFM + b_m * (uint32_t)PF + b_f - bias;
     const typename QuadOf<TV>::type* b = qv + e;
-    const float c0 = bilinear_value(load_fquad(b), af, am);        // plane s
-    const float c1 = bilinear_value(load_fquad(b + PFM), af, am);  // plane s+1
+    const float ax = LAYOUT1 ? am : af, ay = LAYOUT1 ? af : am;
+    const float c0 = bilinear_value(load_fquad(b), ax, ay);        // plane s
+    const float c1 = bilinear_value(load_fquad(b + PFM), ax, ay);  // plane s+1
     return fmaf(as, c1 - c0, c0);
 }
 
@@ -411,11 +414,13 @@ __device__ __forceinline__ void tri_pair_quad(const typename QuadOf<TV>::type* _
     const float4 lo1 = load_fquad(b1);
     const float4 hi1 = load_fquad(b1 + PFM);
     {
-        const float c0 = bilinear_value(lo0, af0, am0), c1 = bilinear_value(hi0, af0, am0);
+        const float ax = R.layout ? am0 : af0, ay = R.layout ? af0 : am0;
+        const float c0 = bilinear_value(lo0, ax, ay), c1 = bilinear_value(hi0, ax, ay);
         if (t0) acc += fmaf(as0, c1 - c0, c0);
     }
     {
-        const float c0 = bilinear_value(lo1, af1, am1), c1 = bilinear_value(hi1, af1, am1);
+        const float ax = R.layout ? am1 : af1, ay = R.layout ? af1 : am1;
+        const float c0 = bilinear_value(lo1, ax, ay), c1 = bilinear_value(hi1, ax, ay);
         if (t1) acc += fmaf(as1, c1 - c0, c0);
     }
 }
@@ -606,26 +611,37 @@ __global__ void __launch_bounds__(256, 6) fwd_quad_kernel(
                 // -ym < bound is ym > -bound, with -bound = fmaf(jf, -D, -Y0)
                 // exactly
                 const float nj = (float)nslab;
-                auto march = [&](auto neg) {
+                auto march = [&](auto neg, auto layout1) {
                     constexpr bool NEG = decltype(neg)::value;
+                    constexpr bool LAYOUT1 = decltype(layout1)::value;
                     const float Ds = NEG ? -D : D, Ys = NEG ? -Y0 : Y0;
                     for (float jf = 1.0f; jf <= nj; jf += 1.0f) {
                         const float bound = fmaf(jf, Ds, Ys);
                         const float ym = fmaf(kf, R.d[1], R.x0[1]);
                         if (kf < kef && (NEG ? ym > bound : ym < bound)) {
-                            acc += tri_sample_quad<TV>(vol, R, kf, ym, PF, PFM, bias);
+                            acc += tri_sample_quad<TV, LAYOUT1>(vol, R, kf, ym, PF, PFM, bias);
                             kf += 1.0f;
                         }
                     }
                 };
-                if (sgn > 0.0f)
-                    march(std::false_type{});
-                else
-                    march(std::true_type{});
+                if (sgn > 0.0f) {
+                    if (layout)
+                        march(std::false_type{}, std::true_type{});
+                    else
+                        march(std::false_type{}, std::false_type{});
+                } else {
+                    if (layout)
+                        march(std::true_type{}, std::true_type{});
+                    else
+                        march(std::true_type{}, std::false_type{});
+                }
             }
         }
-        for (; active && kf < kef; kf += 1.0f)
-            acc += tri_sample_quad<TV>(vol, R, kf, fmaf(kf, R.d[1], R.x0[1]), PF, PFM, bias);
+        for (; active && kf < kef; kf += 1.0f) {
+            const float ym = fmaf(kf, R.d[1], R.x0[1]);
+            acc += layout ? tri_sample_quad<TV, true>(vol, R, kf, ym, PF, PFM, bias)
+                          : tri_sample_quad<TV, false>(vol, R, kf, ym, PF, PFM, bias);
+        }
     }
     if (!inside) return;
     TP* o = proj + ((int64_t)a * c.nv + q) * c.nu + p;
@@ -776,6 +792,61 @@ static bool in_core_bricks(const tigre_geometry* g, tigre_dtype vt)
            e > 0 && (d.n_voxel[0] > e || d.n_voxel[1] > e);
 }
 
+// Whether a projection of na angles takes the column projector
+// (forward_cols.cu): the automatic path with the interpolated projector, where
+// its 8-row warps are full and read near planes, and there are enough of
+// them.  Both sides measured (column / quad kernel, ms):
+//   rows fill the warps: 512^2 x 16 volume, 180 angles: 16 rows 2.13 / 2.17,
+//     24 rows 2.86 / 3.11; 512^2 x 12, 12 rows 1.96 / 1.68; 9 rows 1.53 / 1.34;
+//   neighbouring rows at most 1.9 planes apart at the axis: 512^2 x 64, 180
+//     angles: 40 rows (1.8 planes) 5.14 / 5.19, 32 rows (2.3) 4.60 / 4.28, 24
+//     rows (3.1) 4.16 / 3.33;
+//   enough rays for the chip: 256^3, 256^2 rows: 4 angles 0.40 / 0.46, 2 angles
+//     0.39 / 0.30; 128^3, 128^2, 10 angles 0.151 / 0.144; 512^3, 512^2: 2 angles
+//     1.71 / 1.56, 3 angles 2.30 / 2.73; 64^3, 128^2, 20 angles 0.090 / 0.098.
+constexpr int64_t kColsMinRows = 16, kColsMinAngles = 3, kColsMinRays = 250000;
+constexpr double kColsMaxSpacing = 1.9;
+
+static bool takes_columns(const tigre_geometry* g, int64_t na)
+{
+    const tigre_geometry_desc& d = g->desc;
+    const int64_t nv = d.n_det[1], slots = (nv + 7) / 8 * 8;
+    const double spacing = d.d_det[1] * d.DSO / (d.DSD * d.d_voxel[2]);
+    return g->fwd_path == 0 && g->projector == TIGRE_PROJ_INTERPOLATED && nv >= kColsMinRows &&
+           4 * nv >= 3 * slots && spacing <= kColsMaxSpacing && na >= kColsMinAngles &&
+           d.n_det[0] * nv * na >= kColsMinRays;
+}
+
+// Its launch over the angles [a0, a0 + na): blocks of four neighbouring angles
+// (the groups of the four-angle quad kernel), or of one where there are few
+// (the groups would leave warps empty).
+constexpr int64_t kColsGroupAngles = 8;
+
+template <typename TP>
+static tigre_status run_columns(tigre_geometry* g, const float4* quads, TP* proj, int64_t a0,
+                                int64_t na, int batch, int64_t vol_stride, int64_t proj_stride,
+                                cudaStream_t st)
+{
+    const bool all = a0 == 0 && na == (int64_t)g->angles.size();
+    const int* table = nullptr;
+    int64_t groups = 0;
+    if (na >= kColsGroupAngles) {
+        if (all) {
+            table = (const int*)g->angle_groups[1].ptr;
+            groups = g->n_groups[1];
+        } else {
+            TIGRE_TRY(range_group_table(g, 1, a0, na, &table, &groups));
+        }
+        for (int64_t s = 0; s < groups; s += 65535)
+            TIGRE_TRY(launch_forward_columns<TP>(g, quads, proj, (int)a0, table + 4 * s, 4,
+                                                 std::min<int64_t>(65535, groups - s), batch,
+                                                 vol_stride, proj_stride, st));
+        return TIGRE_OK;
+    }
+    return launch_forward_columns<TP>(g, quads, proj, (int)a0, nullptr, 1, na, batch, vol_stride,
+                                      proj_stride, st);
+}
+
 tigre_status forward_workspace(tigre_geometry* g, tigre_dtype vt, int64_t a0, int64_t na,
                                cudaStream_t st)
 {
@@ -795,6 +866,15 @@ tigre_status forward_workspace(tigre_geometry* g, tigre_dtype vt, int64_t a0, in
         return tma_workspace(g, dtype_size(vt), need);
     }
     const bool use_quad = !siddon && (g->fwd_path == 0 || g->fwd_path >= 3);
+    if (takes_columns(g, na)) {
+        const bool all = a0 == 0 && na == (int64_t)g->angles.size();
+        if (!all && na >= kColsGroupAngles) {
+            const int* table = nullptr;
+            int64_t groups = 0;
+            TIGRE_TRY(range_group_table(g, 1, a0, na, &table, &groups));
+        }
+        return g->vol_qxy.ensure(padded_elems(d) * sizeof(float4));  // one set of quads
+    }
     if (in_core_bricks(g, vt)) {  // the bricks' pixel ranges, before any capture
         const int2* pr = nullptr;
         TIGRE_TRY(brick_pixel_ranges(g, &pr));
@@ -857,6 +937,17 @@ tigre_status forward_impl(tigre_geometry* g, const void* vol, tigre_dtype vt, vo
         DeviceBuffer* bufs[2] = {&g->vol_xy, &g->vol_yx};
         DeviceBuffer* qbufs[2] = {&g->vol_qxy, &g->vol_qyx};
         static_assert(sizeof(Q) == 4 * sizeof(float), "a quad is four FP32 coefficients");
+        if (takes_columns(g, na)) {
+            if (d.n_voxel[2] + 2 * kPad > 65535)
+                return fail(TIGRE_ERR_UNSUPPORTED, "volume too deep for one launch");
+            float4* quads = (float4*)g->vol_qxy.ptr;
+            TIGRE_TRY(build_quad_columns<TV>(d, (const TV*)vol, quads, st));
+            ProfScope prof(kProfForward, st);
+            return dispatch_dtype(pt, [&](auto ptag) -> tigre_status {
+                using TP = decltype(ptag);
+                return run_columns<TP>(g, quads, (TP*)proj, a0, na, 1, 0, 0, st);
+            });
+        }
         for (int l = 0; l < 2; ++l) {
             if (!need[l]) continue;
             if (use_quad)
@@ -938,6 +1029,16 @@ tigre_status forward_impl(tigre_geometry* g, const void* vol, tigre_dtype vt, vo
     });
 }
 
+void batch_quad_layouts(const tigre_geometry* g, bool need[2])
+{
+    if (takes_columns(g, (int64_t)g->angles.size())) {
+        need[0] = true;
+        need[1] = false;
+        return;
+    }
+    needed_layouts(g, 0, (int64_t)g->angles.size(), need);
+}
+
 tigre_status forward_batch_impl(tigre_geometry* g, const void* vols, void* projs, int batch,
                                  tigre_dtype dt, void* const quad[2], cudaStream_t st)
 {
@@ -955,20 +1056,29 @@ tigre_status forward_batch_impl(tigre_geometry* g, const void* vols, void* projs
     needed_layouts(g, 0, na, need);
     const int64_t nvox = d.n_voxel[0] * d.n_voxel[1] * d.n_voxel[2];
     const int64_t pe = (int64_t)padded_elems(d);
+    const bool columns = takes_columns(g, na);
+    if (columns && d.n_voxel[2] + 2 * kPad > 65535)
+        return fail(TIGRE_ERR_UNSUPPORTED, "volume too deep for one launch");
     return dispatch_dtype(dt, [&](auto tag) -> tigre_status {
         using T = decltype(tag);
         using Q = typename QuadOf<T>::type;
-        for (int i = 0; i < batch; ++i)
+        for (int i = 0; i < batch; ++i) {
+            const T* vol = (const T*)vols + i * nvox;
+            if (columns)
+                TIGRE_TRY(build_quad_columns<T>(d, vol, (float4*)quad[0] + i * pe, st));
             for (int l = 0; l < 2; ++l)
-                if (need[l])
-                    TIGRE_TRY(build_quads<T>(d, (const T*)vols + i * nvox, (Q*)quad[l] + i * pe, l,
-                                             st));
+                if (need[l] && !columns)
+                    TIGRE_TRY(build_quads<T>(d, vol, (Q*)quad[l] + i * pe, l, st));
+        }
         FwdBatch bt;
         bt.tiles = tiles;
         bt.vol_stride = pe;
         bt.proj_stride = na * c.nu * c.nv;
         ProfScope prof(kProfForward, st);
         // the automatic path of forward_impl for a full-range projection
+        if (columns)
+            return run_columns<T>(g, (const float4*)quad[0], (T*)projs, 0, na, batch, pe,
+                                  bt.proj_stride, st);
         if (g->auto_angle_group == 2) {
             dim3 grid((unsigned)((c.nu + 15) / 16), (unsigned)g->n_groups[0], (unsigned)(tiles * batch));
             fwd_quad_kernel<T, T, false, false, 2, true><<<grid, dim3(32, 8), 0, st>>>(

@@ -34,19 +34,30 @@ __device__ __forceinline__ void split_floor(float x, int& i, float& f)
     f = __fsub_rn(x, __fsub_rn(m, 8388608.0f));
 }
 
-// Bilinear interpolation of one cell of a plane, as every forward kernel
-// takes it.  With taps a = (f, m), b = (f+1, m), c = (f, m+1), d = (f+1, m+1),
-// the coefficients are (a, b - a, c - a, (d - c) - (b - a)) and the value at
-// fractions (af, am) is a + af (b - a) + am ((c - a) + af ((d - c) - (b - a))),
-// three FMAs.
+// Bilinear interpolation of one cell, x (a detector's columns) first and then
+// y (its rows), as every kernel takes it whatever the memory order it reads.
+// With taps a = (x, y), b = (x+1, y), c = (x, y+1), d = (x+1, y+1), the
+// coefficients are stored as (a, c - a, b - a, (d - c) - (b - a)), so that
+// both x interpolations are one packed FMA on (first, second) halves and the
+// y interpolation a third: value = (a + fx (b - a)) + fy ((c - a) + fx w).
 __host__ __device__ __forceinline__ float4 bilinear_coefficients(float a, float b, float c, float d)
 {
-    const float df = b - a;
-    return make_float4(a, df, c - a, (d - c) - df);
+    const float dx = b - a;
+    return make_float4(a, c - a, dx, (d - c) - dx);
 }
-__device__ __forceinline__ float bilinear_value(const float4& e, float af, float am)
+__device__ __forceinline__ float bilinear_value(const float4& e, float fx, float fy)
 {
-    return fmaf(am, fmaf(af, e.w, e.z), fmaf(af, e.y, e.x));
+    const float2 t = __ffma2_rn(make_float2(fx, fx), make_float2(e.z, e.w), make_float2(e.x, e.y));
+    return fmaf(fy, t.y, t.x);
+}
+
+// The same from the taps of a cell on a layout's (f, m) axes: x is f in
+// layout 0 and m in layout 1.
+__device__ __forceinline__ float bilinear_fm(int layout, float v00, float vf, float vm, float vfm,
+                                             float af, float am)
+{
+    return layout ? bilinear_value(bilinear_coefficients(v00, vm, vf, vfm), am, af)
+                  : bilinear_value(bilinear_coefficients(v00, vf, vm, vfm), af, am);
 }
 
 // The same split with the integer part left biased: b = i + 0x4B000000, the

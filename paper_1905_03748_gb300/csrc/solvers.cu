@@ -733,8 +733,8 @@ tigre_status batch_init(Batch* S, int hist_cap, bool x0_zero)
     TIGRE_TRY(dalloc((unsigned char**)&S->q, B * (size_t)S->m * e, S->st));
     TIGRE_TRY(dalloc((unsigned char**)&S->p, B * (size_t)S->nvox * e, S->st));
     TIGRE_TRY(dalloc((unsigned char**)&S->s, B * (size_t)S->nvox * e, S->st));
-    bool need[2] = {false, false};
-    for (int l : S->g->layout) need[l] = true;
+    bool need[2];
+    batch_quad_layouts(S->g, need);
     for (int l = 0; l < 2; ++l)
         if (need[l]) TIGRE_TRY(dalloc((unsigned char**)&S->quad[l], B * (size_t)S->pe * sizeof(float4), S->st));
     TIGRE_TRY(dalloc((unsigned char**)&S->bpws, B * backward_batch_workspace_bytes(S->g, S->dt),
