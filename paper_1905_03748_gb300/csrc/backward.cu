@@ -94,29 +94,33 @@ template <typename TP> struct ProjTaps<TP, true> {
 // projections (the normaliser V^-1 = A_w^T 1, from the same weights and
 // interpolation) and finish with vol += lambda * num / den (den > 1e-12),
 // clamped at zero when nonneg.
-// Shape (512^3 x 360, one launch).  Plain buffer, 16 voxels per thread at 5
-// blocks per SM (48 registers): matched 51.2 ms, FDK 46.5 ms.  Quad buffer
-// (bilinear coefficients), matched: 16 voxels at 3 blocks 37.4 ms (16 at 4:
-// 37.9; 12 at 6: 41.2; 12 at 5: 40.7; 10 at 6: 39.7; 14 at 5: 44.3; 1024^3 x
-// 180: 142 at 16 / 3 or 4 against 155 at 12 / 6); FDK: 16 voxels at 3 blocks
-// 34.3 ms (16 at 4: 36.5; 12 at 5: 58.0; 8 at 6: 48.5).  SART form (twice the
-// accumulators): plain 16 at 3 blocks 74.2 ms per SIRT pass over 360 angles
-// and 88.1 per OS-SART sweep of 20-angle subsets; quads with 12 voxels at 4
-// blocks 56.4 and 58.9 ms (8 at 6: 58.0 and 61.0; 16 at 3: 57.6 and 61.7).
-template <int MODE, bool SART, bool QUADP>
-constexpr int bp_blocks_per_sm()
+//
+// What bounds it (384^3 x 72, matched, ncu): L1 data pipe 90 %, issue 63 %, FMA
+// pipe 57 %.  A 128-bit warp load takes four wavefronts at least, one per
+// eight lanes, whatever the lanes share (5.3 measured with 8 x 4 tiles).
+//  * Lanes: a warp is a 4 x 8 tile of columns, so eight lanes (4 x 2) span few
+//    detector columns and seldom meet in a bank group.  512^3 x 360 matched /
+//    FDK ms: 32 x 1 37.4 / 33.3, 16 x 2 31.9 / 30.5, 8 x 4 31.0 / 29.6, 4 x 8
+//    30.7 / 29.1; 256^3 x 360 under 384^2 pixels (matched): 5.5, 4.96, 4.91, 4.40.
+//  * Voxels are taken in pairs, as packed FP32 (FFMA2), and a cell's address is
+//    a 32-bit offset from the angle's image: 15.6 warp instructions per 32
+//    voxel-angles (22.3 before; 19.3 with 64-bit addresses, 32.9 ms).
+// Voxels per thread / blocks per SM (registers: 64 at 4 blocks), 512^3 x 360
+// matched / FDK: 16/4 30.7 / 29.1, 16/3 31.7 / 30.0, 12/4 31.2 / 29.5, 8/4 33.7
+// / 30.2, 4/4 42.1 / 34.1.  SART form, SIRT pass 384^3 x 180: 16/3 8.75 ms,
+// 16/4 9.13, 8/4 9.36.  Fewer voxels per thread where the columns alone do not
+// fill the chip (blocks at 16 voxels): 192^3 (1728 blocks) OS-SART sweep 8/4
+// 1.51, 16/3 1.63; 128^3 (512) 8/4 0.182, 16/4 0.188, 4/4 0.214; 64^3 (64) 4/4
+// 0.049, 8/4 0.073, 16/4 0.135.  The line between 8 and 16 lies between the 1728
+// blocks of 192^3 and the 4096 of 256^3 (16/4 4.40, 8/4 4.82).
+// Plain (out-of-core, fewer than four angles) buffers: 16 voxels, 5 or 3 blocks.
+constexpr int kBpLaneX = 4;
+template <bool SART, bool QUADP>
+constexpr int bp_blocks_per_sm(int nz)
 {
-    return !QUADP ? (SART ? 3 : 5) : SART ? 4 : 3;
+    return !QUADP ? (SART ? 3 : 5) : SART && nz == 16 ? 3 : 4;
 }
-template <int MODE, bool SART, bool QUADP>
-constexpr int bp_voxels_per_thread()
-{
-    return !QUADP ? 16 : SART ? 12 : 16;
-}
-static_assert(bp_voxels_per_thread<TIGRE_BP_FDK, false, false>() <= kBpNZ &&
-                  bp_voxels_per_thread<TIGRE_BP_MATCHED, false, true>() <= kBpNZ &&
-                  bp_voxels_per_thread<TIGRE_BP_FDK, false, true>() <= kBpNZ,
-              "the row-band bounds assume chunks of at most kBpNZ planes");
+constexpr int64_t kBpBlocks16 = 2500, kBpBlocks8 = 300;  // blocks at 16 voxels per thread
 
 // Members of a batched launch: blockIdx.z = member * chunks + z chunk; member
 // i reads projections proj_stride elements and writes the volume vol_stride
@@ -127,7 +131,7 @@ struct BpBatch {
 };
 
 template <typename TP, typename TV, int NZ, int MODE, bool SART, bool QUADP, bool BATCH = false>
-__global__ void __launch_bounds__(256, (bp_blocks_per_sm<MODE, SART, QUADP>())) bp_voxel_kernel(
+__global__ void __launch_bounds__(256, (bp_blocks_per_sm<SART, QUADP>(NZ))) bp_voxel_kernel(
                                                        const typename ProjTaps<TP, QUADP>::E* __restrict__ pp,
                                                        TV* __restrict__ vol,
                                                        const BpAngle* __restrict__ params,
@@ -143,8 +147,9 @@ __global__ void __launch_bounds__(256, (bp_blocks_per_sm<MODE, SART, QUADP>())) 
         pp += member * bt.proj_stride;
         vol += member * bt.vol_stride;
     }
-    const int x = blockIdx.x * 32 + threadIdx.x;
-    const int y = blockIdx.y * 8 + threadIdx.y;
+    constexpr int LX = kBpLaneX, LY = 32 / LX;
+    const int x = blockIdx.x * 32 + ((int)threadIdx.y % (32 / LX)) * LX + (int)threadIdx.x % LX;
+    const int y = blockIdx.y * 8 + ((int)threadIdx.y / (32 / LX)) * LY + (int)threadIdx.x / LX;
     const int zb = c.z_first + ((int)blockIdx.z - member * bt.chunks) * NZ;
     if (x >= c.nx || y >= c.ny) return;
     const float X = fmaf((float)x, c.dx, c.x0);
@@ -154,19 +159,21 @@ __global__ void __launch_bounds__(256, (bp_blocks_per_sm<MODE, SART, QUADP>())) 
     const int64_t PA = (int64_t)PU * c.PV;
     const float pu_hi = (float)c.nu + 0.5f;
     const float pv_off = c.pv_off + (float)c.pv_lo;
-    // a row's element offset from split_bits parts: (b - 0x4B000000) PU, one
-    // multiply-add modulo 2^32
-    const uint32_t row_bias = 0x4B000000u * (uint32_t)PU;
+    const uint32_t pitch = (uint32_t)(PU * sizeof(typename ProjTaps<TP, QUADP>::E));
+    const float pv_in_lo = (float)c.pv_lo, pv_in_hi = (float)(c.pv_lo + c.nv - 1);
 
-    float acc[NZ];
-    float nrm[SART ? NZ : 1];
+    float2 half2 = make_float2(8388607.5f, 8388607.5f), two23 = make_float2(8388608.0f, 8388608.0f);
+    static_assert(NZ % 2 == 0, "voxels are taken in pairs");
+    float2 acc[NZ / 2];
+    float2 nrm[SART ? NZ / 2 : 1];
 #pragma unroll
-    for (int k = 0; k < NZ; ++k) acc[k] = 0.0f;
+    for (int k = 0; k < NZ / 2; ++k) acc[k] = make_float2(0.0f, 0.0f);
 #pragma unroll
-    for (int k = 0; k < (SART ? NZ : 1); ++k) nrm[k] = 0.0f;
+    for (int k = 0; k < (SART ? NZ / 2 : 1); ++k) nrm[k] = make_float2(0.0f, 0.0f);
 
     for (int a = 0; a < na; ++a) {
-        const BpAngle A = params[a_first + a];
+        const float4 Av = __ldg((const float4*)(params + a_first + a));
+        const BpAngle A{Av.x, Av.y, Av.z, Av.w};
         const float s = fmaf(X, A.c, Y * A.s);
         const float inv_den = 1.0f / (c.DSO - s);
         const float mag = c.DSD * inv_den;
@@ -176,15 +183,21 @@ __global__ void __launch_bounds__(256, (bp_blocks_per_sm<MODE, SART, QUADP>())) 
         int ip;
         float fu;
         split_floor(pu, ip, fu);
-        const typename ProjTaps<TP, QUADP>::E* col = pp + (int64_t)a * PA + ip;
+        // split_bits' 0x4B000000 leaves the row offset here, once per column:
+        // a cell's address is then one wide multiply-add
+        const char* abase = (const char*)(pp + (int64_t)a * PA);
+        const uint32_t cofs = (uint32_t)ip * (uint32_t)sizeof(*pp) - 0x4B000000u * pitch;
         // Padded row coordinate of voxel k: within [2, PV - 2) by the
         // host-side bound on the volume's shadow.
         const float pv0 = fmaf(Zb * mag, c.inv_dv, pv_off);
         const float dpv = c.dz * mag * c.inv_dv;
         float tu = 0.0f;  // bilinear weight of the all-ones image along u
-        if (SART)
+        bool inner = true;  // and along v: 1 where every cell lies on the detector
+        if (SART) {
             tu = ((unsigned)(ip - kPad) < (unsigned)c.nu ? 1.0f - fu : 0.0f) +
                  ((unsigned)(ip - kPad + 1) < (unsigned)c.nu ? fu : 0.0f);
+            inner = pv0 >= pv_in_lo && fmaf((float)(NZ - 1), dpv, pv0) <= pv_in_hi;
+        }
         // matched: voxel k's weight w |source - voxel| is taken as
         // sqrt(u) = u rsqrt(u) with u = (w Z)^2 + w^2 |(ex, ey)|^2, one
         // multiply fewer per voxel than w (l2 rsqrt(l2))
@@ -199,26 +212,41 @@ __global__ void __launch_bounds__(256, (bp_blocks_per_sm<MODE, SART, QUADP>())) 
             wdz = w * c.dz;
             wZb = w * Zb;
         }
+        // voxels two at a time, as packed FP32 pairs
 #pragma unroll
-        for (int k = 0; k < NZ; ++k) {
-            uint32_t bq;
-            float fv;
-            split_bits(fmaf((float)k, dpv, pv0), bq, fv);
-            // the cell of columns ip, ip + 1 and rows iq, iq + 1 (iq = bq - 0x4B000000)
-            const auto* cell = col + (bq * (uint32_t)PU - row_bias);
-            const float val = bilinear_value(ProjTaps<TP, QUADP>::load(cell, PU), fu, fv);
-            float wk = w;
-            if (MODE != TIGRE_BP_FDK) {
-                const float Zw = fmaf((float)k, wdz, wZb);
-                const float u2 = fmaf(Zw, Zw, w2lxy);
-                wk = u2 * rsqrt_sfu(u2);
+        for (int k = 0; k < NZ; k += 2) {
+            const float2 pv = make_float2(fmaf((float)k, dpv, pv0), fmaf((float)(k + 1), dpv, pv0));
+            const float2 m = __fadd2_rn(pv, half2);
+            const float2 fv = sub2(pv, sub2(m, two23));
+            const uint32_t b0 = __float_as_uint(m.x), b1 = __float_as_uint(m.y);
+            // the cell of columns ip, ip + 1 and rows iq, iq + 1 (iq = b - 0x4B000000)
+            using E = typename ProjTaps<TP, QUADP>::E;
+            const E *cell0, *cell1;
+            if (QUADP) {
+                cell0 = (const E*)(abase + (b0 * pitch + cofs));
+                cell1 = (const E*)(abase + (b1 * pitch + cofs));
+            } else {  // images of any size
+                cell0 = (const E*)abase + (int64_t)(b0 - 0x4B000000u) * PU + ip;
+                cell1 = (const E*)abase + (int64_t)(b1 - 0x4B000000u) * PU + ip;
             }
-            acc[k] = fmaf(wk, val, acc[k]);
+            const float4 e0 = ProjTaps<TP, QUADP>::load(cell0, PU), e1 = ProjTaps<TP, QUADP>::load(cell1, PU);
+            const float2 val = make_float2(bilinear_value(e0, fu, fv.x), bilinear_value(e1, fu, fv.y));
+            float2 wk = make_float2(w, w);
+            if (MODE != TIGRE_BP_FDK) {
+                const float2 Zw = make_float2(fmaf((float)k, wdz, wZb), fmaf((float)(k + 1), wdz, wZb));
+                const float2 u2 = __ffma2_rn(Zw, Zw, make_float2(w2lxy, w2lxy));
+                wk = __fmul2_rn(u2, make_float2(rsqrt_sfu(u2.x), rsqrt_sfu(u2.y)));
+            }
+            acc[k / 2] = __ffma2_rn(wk, val, acc[k / 2]);
             if (SART) {
-                const uint32_t qq = bq - (0x4B000000u + (uint32_t)c.pv_lo);
-                const float tv = (qq < (unsigned)c.nv ? 1.0f - fv : 0.0f) +
-                                 (qq + 1u < (unsigned)c.nv ? fv : 0.0f);
-                nrm[k] = fmaf(wk, tu * tv, nrm[k]);
+                float2 t = make_float2(tu, tu);
+                if (!inner) {
+                    const uint32_t q0 = b0 - (0x4B000000u + (uint32_t)c.pv_lo);
+                    const uint32_t q1 = b1 - (0x4B000000u + (uint32_t)c.pv_lo);
+                    t.x *= (q0 < (unsigned)c.nv ? 1.0f - fv.x : 0.0f) + (q0 + 1u < (unsigned)c.nv ? fv.x : 0.0f);
+                    t.y *= (q1 < (unsigned)c.nv ? 1.0f - fv.y : 0.0f) + (q1 + 1u < (unsigned)c.nv ? fv.y : 0.0f);
+                }
+                nrm[k / 2] = __ffma2_rn(wk, t, nrm[k / 2]);
             }
         }
     }
@@ -227,15 +255,16 @@ __global__ void __launch_bounds__(256, (bp_blocks_per_sm<MODE, SART, QUADP>())) 
         const int z = zb + k;
         if (z < c.z_end) {
             TV* o = vol + ((int64_t)(z - c.z_out0) * c.ny + y) * c.nx + x;
+            const float num = k & 1 ? acc[k / 2].y : acc[k / 2].x;
             if (SART) {
-                const float den = nrm[k];
+                const float den = k & 1 ? nrm[k / 2].y : nrm[k / 2].x;
                 float v = to_f32<TV>(*o);
-                if (den > 1e-12f) v = fmaf(lambda, acc[k] / den, v);
+                if (den > 1e-12f) v = fmaf(lambda, num / den, v);
                 if (nonneg) v = fmaxf(v, 0.0f);
                 *o = from_f32<TV>(v);
             } else {
                 const float prev = accumulate ? to_f32<TV>(*o) : 0.0f;
-                *o = from_f32<TV>(prev + acc[k]);
+                *o = from_f32<TV>(prev + num);
             }
         }
     }
@@ -440,6 +469,13 @@ static bool bp_reads_quads(tigre_bp_weight w)
     return w == TIGRE_BP_MATCHED || w == TIGRE_BP_FDK;
 }
 
+// Quad launches address an angle's image in 32 bits; larger images (more than
+// 2^28 padded pixels) are read from the plain buffer.
+static bool bp_quads_addressable(const BpConst& c)
+{
+    return (int64_t)c.PU * c.PV < ((int64_t)1 << 28);
+}
+
 tigre_status backward_workspace(tigre_geometry* g, tigre_dtype pt, tigre_bp_weight w, int64_t a0,
                                 int64_t na)
 {
@@ -491,10 +527,16 @@ static tigre_status run_voxel_bp(tigre_geometry* g, const BpConst& c, const TP* 
     const dim3 block(32, 8);
     ProfScope prof(kProfBackproject, st);
     // One kernel instance: MODE and SART fixed, NZ voxels per thread.
-    auto launch = [&](auto mode, auto sart_tag) -> tigre_status {
+    // Voxels per thread from one member's blocks, so that a problem's numbers
+    // are the same alone and in a batch.
+    const int64_t cols = (int64_t)((c.nx + 31) / 32) * ((c.ny + 7) / 8);
+    const int64_t blocks16 = cols * ((c.z_end - c.z_first + 15) / 16);
+    // One kernel instance: MODE and SART fixed, NZ voxels per thread.
+    auto launch_nz = [&](auto mode, auto sart_tag, auto nz) -> tigre_status {
         constexpr int M = decltype(mode)::value;
         constexpr bool S = decltype(sart_tag)::value;
-        constexpr int NZ = bp_voxels_per_thread<M, S, QUADP>();
+        constexpr int NZ = decltype(nz)::value;
+        static_assert(NZ <= kBpNZ, "the row-band bounds assume chunks of at most kBpNZ planes");
         const int chunks = (c.z_end - c.z_first + NZ - 1) / NZ;
         dim3 grid((unsigned)((c.nx + 31) / 32), (unsigned)((c.ny + 7) / 8),
                   (unsigned)((int64_t)chunks * batch));
@@ -506,18 +548,27 @@ static tigre_status run_voxel_bp(tigre_geometry* g, const BpConst& c, const TP* 
             bt.proj_stride = (int64_t)pelems;
             bt.vol_stride = (int64_t)c.nx * c.ny * c.nz;
         }
-        // Single launches take the instance without member offsets (512^3 x
-        // 360: FDK 36.3 vs 41.6 ms, matched 40.8 vs 41.2), except the SART
-        // update, whose instance with them compiles to a faster kernel (SIRT
-        // pass 58.0 vs 59.0 ms); with one member the offsets are zero.
-        constexpr bool kSingle = !S;  // SART: the instance with offsets only
-        if (!kSingle || batch > 1)
-            bp_voxel_kernel<TP, TV, NZ, M, S, QUADP, true><<<grid, block, 0, st>>>(
-                pp, vol, params, c, (int)a0, (int)na, S ? 0 : accumulate, lambda, nonneg, bt);
-        else if constexpr (kSingle)
-            bp_voxel_kernel<TP, TV, NZ, M, S, QUADP><<<grid, block, 0, st>>>(
-                pp, vol, params, c, (int)a0, (int)na, accumulate, lambda, nonneg, bt);
+        // (single launches take the instance without member offsets: FDK at
+        // 512^3 x 360 33.3 ms against 37.8 with them)
+        if constexpr (QUADP && !S) {
+            if (batch > 1) {
+                bp_voxel_kernel<TP, TV, NZ, M, S, QUADP, true><<<grid, block, 0, st>>>(
+                    pp, vol, params, c, (int)a0, (int)na, accumulate, lambda, nonneg, bt);
+                return TIGRE_OK;
+            }
+        }
+        bp_voxel_kernel<TP, TV, NZ, M, S, QUADP><<<grid, block, 0, st>>>(
+            pp, vol, params, c, (int)a0, (int)na, S ? 0 : accumulate, lambda, nonneg, bt);
         return TIGRE_OK;
+    };
+    auto launch = [&](auto mode, auto sart_tag) -> tigre_status {
+        if constexpr (QUADP) {
+            if (blocks16 < kBpBlocks8)
+                return launch_nz(mode, sart_tag, std::integral_constant<int, 4>{});
+            if (blocks16 < kBpBlocks16)
+                return launch_nz(mode, sart_tag, std::integral_constant<int, 8>{});
+        }
+        return launch_nz(mode, sart_tag, std::integral_constant<int, 16>{});
     };
     using Fdk = std::integral_constant<int, TIGRE_BP_FDK>;
     using Matched = std::integral_constant<int, TIGRE_BP_MATCHED>;
@@ -550,7 +601,7 @@ tigre_status launch_voxel_bp(tigre_geometry* g, const TP* proj, TV* vol, int64_t
         c.z_out0 = z_out0;
         bp_slab_band(c, d, z_first, z_end);
     }
-    if (!bp_reads_quads(w))
+    if (!bp_reads_quads(w) || !bp_quads_addressable(c))
         return run_voxel_bp<TP, TV, false>(g, c, proj, vol, a0, na, w, accumulate, st, sart,
                                            lambda, nonneg);
     if (z_end < 0)
@@ -591,6 +642,13 @@ tigre_status backward_batch_impl(tigre_geometry* g, const void* projs, void* vol
     const int64_t na = (int64_t)g->angles.size();
     return dispatch_dtype(dt, [&](auto tag) -> tigre_status {
         using T = decltype(tag);
+        if (!bp_quads_addressable(c)) {
+            for (int i = 0; i < batch; ++i)
+                TIGRE_TRY((run_voxel_bp<T, T, false>(
+                    g, c, (const T*)projs + i * na * c.nu * c.nv,
+                    (T*)vols + i * (int64_t)c.nx * c.ny * c.nz, 0, na, w, 0, st, false, 0.0f, 0, 1, ws)));
+            return TIGRE_OK;
+        }
         return run_voxel_bp<T, T, true>(g, c, (const T*)projs, (T*)vols, 0, na, w, 0, st, false,
                                         0.0f, 0, batch, ws);
     });

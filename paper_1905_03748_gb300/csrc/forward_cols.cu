@@ -97,17 +97,6 @@ __device__ __forceinline__ void load_cell(const float4* __restrict__ q, uint32_t
     cur = e;
 }
 
-// a - b on both halves, each rounded to nearest.
-__device__ __forceinline__ float2 sub2(float2 a, float2 b)
-{
-    float2 r;
-    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
-        "sub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-
 struct ColGeom {
     uint32_t SX, SY;  // quads between x and y neighbours
     uint32_t bias;    // of an element index built from split_bits parts

@@ -34,6 +34,17 @@ __device__ __forceinline__ void split_floor(float x, int& i, float& f)
     f = __fsub_rn(x, __fsub_rn(m, 8388608.0f));
 }
 
+// a - b on both halves, each rounded to nearest.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+        "sub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
 // Bilinear interpolation of one cell, x (a detector's columns) first and then
 // y (its rows), as every kernel takes it whatever the memory order it reads.
 // With taps a = (x, y), b = (x+1, y), c = (x, y+1), d = (x+1, y+1), the
