@@ -34,6 +34,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "forward_cols.cuh"
 #include "quad.cuh"
 #include "ray.cuh"
 
@@ -476,6 +477,13 @@ static bool bp_quads_addressable(const BpConst& c)
     return (int64_t)c.PU * c.PV < ((int64_t)1 << 28);
 }
 
+// Whether an exact adjoint takes the column scatter (adjoint_cols.cu), by the
+// forward projector's rule.
+static bool adjoint_takes_columns(const tigre_geometry* g, int64_t na)
+{
+    return g->projector == TIGRE_PROJ_INTERPOLATED && column_warps_pay(g, na);
+}
+
 tigre_status backward_workspace(tigre_geometry* g, tigre_dtype pt, tigre_bp_weight w, int64_t a0,
                                 int64_t na)
 {
@@ -485,6 +493,7 @@ tigre_status backward_workspace(tigre_geometry* g, tigre_dtype pt, tigre_bp_weig
     const tigre_geometry_desc& d = g->desc;
     if (w == TIGRE_BP_EXACT_ADJOINT) {
         if (padded_elems(d) >= (size_t)INT32_MAX) return TIGRE_OK;  // refused by the operator
+        if (adjoint_takes_columns(g, na)) return g->adj_xy.ensure(padded_elems(d) * sizeof(float4));
         bool need[2] = {false, false};
         for (int64_t a = a0; a < a0 + na; ++a) need[g->layout[(size_t)a]] = true;
         DeviceBuffer* bufs[2] = {&g->adj_xy, &g->adj_yx};
@@ -699,6 +708,15 @@ static tigre_status launch_adjoint(tigre_geometry* g, const TP* proj, TV* vol, i
     if (padded_elems(d) >= (size_t)INT32_MAX)
         return fail(TIGRE_ERR_UNSUPPORTED, "exact adjoint needs (nx+4)(ny+4)(nz+4) < 2^31");
     const FwdConst c = make_fwd_const(g);
+    if (adjoint_takes_columns(g, na)) {
+        const size_t quads = padded_elems(d) * sizeof(float4);
+        TIGRE_TRY(g->adj_xy.ensure(quads));
+        g->adj_xy.tag = 0;
+        TIGRE_CUDA(cudaMemsetAsync(g->adj_xy.ptr, 0, quads, st));
+        ProfScope prof(kProfAdjoint, st);
+        return launch_adjoint_columns<TP, TV>(g, proj, (float4*)g->adj_xy.ptr, vol, a0, na,
+                                              accumulate, st);
+    }
     bool need[2] = {false, false};
     for (int64_t a = a0; a < a0 + na; ++a) need[g->layout[(size_t)a]] = true;
     DeviceBuffer* bufs[2] = {&g->adj_xy, &g->adj_yx};

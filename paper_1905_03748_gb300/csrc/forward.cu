@@ -807,14 +807,18 @@ static bool in_core_bricks(const tigre_geometry* g, tigre_dtype vt)
 constexpr int64_t kColsMinRows = 16, kColsMinAngles = 3, kColsMinRays = 250000;
 constexpr double kColsMaxSpacing = 1.9;
 
-static bool takes_columns(const tigre_geometry* g, int64_t na)
+bool column_warps_pay(const tigre_geometry* g, int64_t na)
 {
     const tigre_geometry_desc& d = g->desc;
     const int64_t nv = d.n_det[1], slots = (nv + 7) / 8 * 8;
     const double spacing = d.d_det[1] * d.DSO / (d.DSD * d.d_voxel[2]);
-    return g->fwd_path == 0 && g->projector == TIGRE_PROJ_INTERPOLATED && nv >= kColsMinRows &&
-           4 * nv >= 3 * slots && spacing <= kColsMaxSpacing && na >= kColsMinAngles &&
-           d.n_det[0] * nv * na >= kColsMinRays;
+    return nv >= kColsMinRows && 4 * nv >= 3 * slots && spacing <= kColsMaxSpacing &&
+           na >= kColsMinAngles && d.n_det[0] * nv * na >= kColsMinRays;
+}
+
+static bool takes_columns(const tigre_geometry* g, int64_t na)
+{
+    return g->fwd_path == 0 && g->projector == TIGRE_PROJ_INTERPOLATED && column_warps_pay(g, na);
 }
 
 // Its launch over the angles [a0, a0 + na): blocks of four neighbouring angles
