@@ -10,8 +10,8 @@
 //      distance weight (DSO/(DSO-s))^2, each angle times half its angular
 //      weight (half the angle between its neighbours on the circle).
 //
-// Step 1, 2 and the angular factor run in one kernel (one block per detector
-// row, the row in shared memory); step 3 is the voxel-driven backprojector.
+// Step 1, 2 and the angular factor run in one kernel (a block takes 8, 4 or 1
+// detector rows into shared memory); step 3 is the voxel-driven backprojector.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -54,6 +54,92 @@ __global__ void __launch_bounds__(256) fdk_filter_kernel(const TP* __restrict__ 
             acc = fmaf(h_odd[i], l + r, acc);
         }
         dst[p] = wa * acc;
+    }
+}
+
+// The same filter for R rows of one angle per block, as two dense convolutions:
+// an even output sums odd inputs only and an odd output even ones, so the rows
+// are split by parity.  With G[d] = h at offset 2d + 1 (G[-d - 1] = G[d]), the
+// outputs are
+//   out[2m + 1] = h0 y[2m + 1] + sum_n G[m - n] y[2n],
+//   out[2m]     = h0 y[2m]     + sum_n G[m - n - 1] y[2n + 1].
+// A thread makes four neighbouring outputs of one parity for all R rows: per
+// four inputs it reads two float4 of G and one of each row (the same for the
+// whole warp) for 16 R multiply-adds, so it is bound by FMA where one output
+// per thread was bound by two shared-memory loads per multiply-add.
+// 509 x 397 x 361 (FP16 in): 6.11 -> 0.95 ms.
+constexpr int kFdkThreads = 128;
+
+template <typename TP, int R>
+__global__ void __launch_bounds__(kFdkThreads) fdk_filter_rows_kernel(
+    const TP* __restrict__ proj, float* __restrict__ out, const float* __restrict__ h_odd,
+    const float* __restrict__ ang_w, int nu, int nv, float h0, float u0, float du, float v0,
+    float dv, float dsd2)
+{
+    extern __shared__ float4 shared4[];
+    // half rows of H values (a multiple of 4, zero beyond the detector):
+    // rows[parity][r][H], then G[-H .. H + 4)
+    const int H = ((nu + 1) / 2 + 3) & ~3;
+    float* rows = (float*)shared4;
+    float* G = rows + 2 * R * H + H;  // (G[0] here)
+    const int q0 = blockIdx.x * R, a = blockIdx.y;
+    for (int i = threadIdx.x; i < R * 2 * H; i += kFdkThreads) {
+        const int r = i / (2 * H), p = i - r * 2 * H, q = q0 + r;
+        float y = 0.0f;
+        if (q < nv && p < nu) {
+            const float v = fmaf((float)q, dv, v0), u = fmaf((float)p, du, u0);
+            y = to_f32<TP>(proj[((int64_t)a * nv + q) * nu + p]) * sqrtf(dsd2) *
+                rsqrtf(dsd2 + u * u + v * v);
+        }
+        rows[((p & 1) * R + r) * H + (p >> 1)] = y;
+    }
+    const int nh = nu / 2;  // odd offsets 1, 3, ... below nu
+    for (int d = (int)threadIdx.x - H; d < H + 4; d += kFdkThreads) {
+        const int i = d >= 0 ? d : -d - 1;
+        G[d] = i < nh ? h_odd[i] : 0.0f;
+    }
+    __syncthreads();
+    const float wa = ang_w[a];
+    const int quads = H / 4;
+    for (int t = threadIdx.x; t < 2 * quads; t += kFdkThreads) {
+        const int par = t >= quads, m = 4 * (t - par * quads);  // outputs 2 (m + i) + par
+        const float* in = rows + (1 - par) * R * H;             // inputs of the other parity
+        const float* own = rows + par * R * H;
+        float acc[R][4];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[r][i] = 0.0f;
+        for (int n = 0; n < H; n += 4) {
+            // the centre tap enters between its neighbours, which nearly cancel
+            // it on smooth rows: the far taps then add to small sums
+            if (n == m)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[r][i] = fmaf(h0, own[r * H + m + i], acc[r][i]);
+            const float4 lo = *(const float4*)(G + m - n - 4), hi = *(const float4*)(G + m - n);
+            const float g[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float4 y = *(const float4*)(in + r * H + n);
+                // g[4 + i - j] = G[(m + i) - (n + j)], one earlier for even outputs
+                const float yj[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        acc[r][i] = fmaf(par ? g[4 + i - j] : g[3 + i - j], yj[j], acc[r][i]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (q0 + r < nv) {
+                float* dst = out + ((int64_t)a * nv + q0 + r) * nu;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (2 * (m + i) + par < nu) dst[2 * (m + i) + par] = wa * acc[r][i];
+            }
     }
 }
 
@@ -121,6 +207,22 @@ tigre_status fdk_impl(tigre_geometry* g, const void* proj, tigre_dtype pt, void*
         const size_t smem = sizeof(float) * (size_t)nu;
         status = dispatch_dtype(pt, [&](auto tag) -> tigre_status {
             using TP = decltype(tag);
+            // Blocks of 8 rows up to 2048 columns (73 KB: three per SM), of 4
+            // up to 8192 (164 KB); longer rows one by one.
+            auto rows = [&](auto kern, int R) -> tigre_status {
+                const int H = ((nu + 1) / 2 + 3) & ~3;
+                const int bytes = (int)sizeof(float) * (2 * R * H + 2 * H + 4);
+                if (bytes > 48 * 1024)
+                    TIGRE_CUDA(cudaFuncSetAttribute(
+                        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+                kern<<<dim3((unsigned)((nv + R - 1) / R), (unsigned)na), kFdkThreads, bytes, st>>>(
+                    (const TP*)proj, filt, dtab, dtab + (nu / 2 + 1), nu, nv, h0, u0,
+                    (float)d.d_det[0], v0, (float)d.d_det[1], (float)(d.DSD * d.DSD));
+                TIGRE_LAUNCHED("fdk_filter_rows_kernel");
+                return TIGRE_OK;
+            };
+            if (nu <= 2048) return rows(fdk_filter_rows_kernel<TP, 8>, 8);
+            if (nu <= 8192) return rows(fdk_filter_rows_kernel<TP, 4>, 4);
             if (smem > 48 * 1024)
                 TIGRE_CUDA(cudaFuncSetAttribute(fdk_filter_kernel<TP>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
