@@ -271,40 +271,43 @@ __global__ void __launch_bounds__(256, (bp_blocks_per_sm<SART, QUADP>(NZ))) bp_v
     }
 }
 
-template <typename TP>
-__device__ __forceinline__ TP pix_or_zero(const TP* row, int p, int nu)
-{
-    return (unsigned)p < (unsigned)nu ? row[p] : from_f32<TP>(0.0f);
-}
-
 // Write the whole zero-bordered buffer of one angle range: with
 // Z(r, c) = y[a][r - pv_lo][c - 2] (zero outside the detector), the plain
 // buffer holds out[a][r][c] = Z(r, c), the quad buffer the FP32 bilinear
 // coefficients of the cell (Z(r, c), Z(r, c+1), Z(r+1, c), Z(r+1, c+1)).
+// A thread makes one column of four rows, so the taps of five rows are in
+// flight together (one element per thread, rows shorter than its 256-thread
+// block: 512^3 x 360 495 -> 289 us, 360 x 256^2 BF16 149 -> 73).
+constexpr int kPadRows = 4;
 template <typename TP, bool QUADP>
-__global__ void pad_proj_kernel(const TP* __restrict__ in,
-                                typename ProjTaps<TP, QUADP>::E* __restrict__ out, int nu, int nv,
-                                int PU, int PV, int pv_lo)
+__global__ void __launch_bounds__(256) pad_proj_kernel(
+    const TP* __restrict__ in, typename ProjTaps<TP, QUADP>::E* __restrict__ out, int nu, int nv,
+    int PU, int PV, int pv_lo)
 {
-    const int r = blockIdx.y, a = blockIdx.z;
-    const int q = r - pv_lo;
-    typename ProjTaps<TP, QUADP>::E* dst = out + ((int64_t)a * PV + r) * PU;
-    const TP* row0 = in + ((int64_t)a * nv + q) * nu;
-    const TP* row1 = row0 + nu;
-    const bool in0 = (unsigned)q < (unsigned)nv, in1 = (unsigned)(q + 1) < (unsigned)nv;
-    const TP z = from_f32<TP>(0.0f);
-    for (int col = blockIdx.x * blockDim.x + threadIdx.x; col < PU; col += gridDim.x * blockDim.x) {
-        const int p = col - kPad;
-        const TP a00 = in0 ? pix_or_zero(row0, p, nu) : z;
-        if constexpr (!QUADP) {
-            dst[col] = a00;
-        } else {
-            const TP a01 = in0 ? pix_or_zero(row0, p + 1, nu) : z;
-            const TP a10 = in1 ? pix_or_zero(row1, p, nu) : z;
-            const TP a11 = in1 ? pix_or_zero(row1, p + 1, nu) : z;
-            dst[col] = bilinear_coefficients(to_f32<TP>(a00), to_f32<TP>(a01), to_f32<TP>(a10),
-                                             to_f32<TP>(a11));
-        }
+    const int col = blockIdx.x * 64 + threadIdx.x, a = blockIdx.z;
+    const int r0 = (blockIdx.y * 4 + threadIdx.y) * kPadRows;
+    if (col >= PU) return;
+    const int p = col - kPad;
+    const TP* img = in + (int64_t)a * nv * nu;
+    auto tap = [&](int r, int c) -> float {  // Z(r, c + 2)
+        const int q = r - pv_lo;
+        return (unsigned)q < (unsigned)nv && (unsigned)c < (unsigned)nu
+                   ? to_f32<TP>(img[(int64_t)q * nu + c]) : 0.0f;
+    };
+    float left[kPadRows + 1], right[kPadRows + 1];
+#pragma unroll
+    for (int i = 0; i <= kPadRows; ++i) {
+        left[i] = tap(r0 + i, p);
+        right[i] = QUADP ? tap(r0 + i, p + 1) : 0.0f;
+    }
+    typename ProjTaps<TP, QUADP>::E* dst = out + ((int64_t)a * PV + r0) * PU + col;
+#pragma unroll
+    for (int i = 0; i < kPadRows; ++i) {
+        if (r0 + i >= PV) return;
+        if constexpr (QUADP)
+            dst[(int64_t)i * PU] = bilinear_coefficients(left[i], right[i], left[i + 1], right[i + 1]);
+        else
+            dst[(int64_t)i * PU] = from_f32<TP>(left[i]);
     }
 }
 
@@ -526,8 +529,9 @@ static tigre_status run_voxel_bp(tigre_geometry* g, const BpConst& c, const TP* 
     // a batch's projections are consecutive angle blocks of one long buffer
     for (int64_t s = 0; s < na * batch; s += 65535) {
         const int64_t cnt = std::min<int64_t>(65535, na * batch - s);
-        dim3 grid((unsigned)((c.PU + 255) / 256), (unsigned)c.PV, (unsigned)cnt);
-        pad_proj_kernel<TP, QUADP><<<grid, 256, 0, st>>>(proj + s * (int64_t)c.nu * c.nv,
+        dim3 grid((unsigned)((c.PU + 63) / 64), (unsigned)((c.PV + 4 * kPadRows - 1) / (4 * kPadRows)),
+                  (unsigned)cnt);
+        pad_proj_kernel<TP, QUADP><<<grid, dim3(64, 4), 0, st>>>(proj + s * (int64_t)c.nu * c.nv,
                                                    pp + s * (int64_t)c.PU * c.PV, c.nu, c.nv,
                                                    c.PU, c.PV, c.pv_lo);
         TIGRE_LAUNCHED("pad_proj_kernel");
