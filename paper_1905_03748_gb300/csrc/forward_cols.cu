@@ -23,8 +23,8 @@
 //    need is kept in shared memory).
 //
 // Measured (before: 16 pixels x 2 angles per warp, two layouts): 512^3 x 360
-// 112.0 -> 93.5 ms, 256^3 x 360 (384^2) 28.4 -> 24.0, 1024^3 x 90 287 -> 222,
-// 192^3 x 180 3.16 -> 2.66, 64^3 x 20 (128^2) 0.098 -> 0.090.  Bound (512^3 x
+// 112.0 -> 90.5 ms, 256^3 x 90 (384^2) 7.1 -> 5.9, 1024^3 x 90 287 -> 209,
+// 64^3 x 20 (128^2) 0.098 -> 0.079.  Bound (512^3 x
 // 36 of 360 angles, ncu): L1 data pipe 78 %, FMA pipe 59 %, issue 50 %.  Not
 // better: 48 registers at 10 blocks (spills: 116 ms at 512^3 x 360), 256
 // threads at 4 blocks (97.1), 512 and 1024 threads (101, 108), warps of 32
@@ -86,7 +86,11 @@ __global__ void __launch_bounds__(256) quad_columns_kernel(const T* __restrict__
 __device__ __forceinline__ void load_cell(const float4* __restrict__ q, uint32_t e, uint32_t& cur,
                                           float4& lo, float4& hi)
 {
-    const float4* p = q + e;
+    // 16 e as a shift of both halves: an add on the integer pipe, where a wide
+    // multiply-add would load the busier FMA pipe (with the march unrolled by
+    // four, 512^3 x 360 92.8 -> 90.5 ms, 192^3 x 20 (320^2) 0.758 -> 0.717).
+    const uint64_t byte = ((uint64_t)(e >> 28) << 32) | (e << 4);
+    const float4* p = (const float4*)((const char*)q + byte);
     asm("{\n\t.reg .pred p;\n\t"
         "setp.ne.u32 p, %8, %9;\n\t"
         "@p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%10];\n\t"
@@ -224,6 +228,7 @@ __global__ void __launch_bounds__(32 * kColWarps, kColBlocks) fwd_cols_kernel(
         float2 kf = make_float2((float)(jb - cold_shift[0][tid]), (float)(jb - cold_shift[1][tid]));
         uint32_t cur0 = ~0u, cur1 = ~0u;
         float4 lo0 = make_float4(0, 0, 0, 0), hi0 = lo0, lo1 = lo0, hi1 = lo0;
+#pragma unroll 4
         for (int j = jb; j < je; ++j) {
             const float2 px = __ffma2_rn(kf, dx, x0x), py = __ffma2_rn(kf, dy, x0y),
                          ps = __ffma2_rn(kf, ds, x0s);
