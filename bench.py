@@ -36,7 +36,9 @@ UNIT = "Gvoxel*angles/s"
 FLOPS_PER_SAMPLE = 22  # trilinear interpolation: 7 lerps x 3 flops + 1 accumulation
 L1_BYTES_PER_SAMPLE = 32  # the eight FP32 taps a trilinear sample gathers
 L1_BYTES_PER_VOXEL_ANGLE = 16  # the four FP32 taps a backprojected voxel-angle gathers
-KERNEL_SOURCES = ["paper_1905_03748_gb300/csrc/forward.cu", "paper_1905_03748_gb300/csrc/ray.cuh",
+KERNEL_SOURCES = ["paper_1905_03748_gb300/csrc/forward_cols.cu",
+                  "paper_1905_03748_gb300/csrc/forward_cols.cuh",
+                  "paper_1905_03748_gb300/csrc/ray.cuh",
                   "paper_1905_03748_gb300/csrc/quad.cuh"]
 BP_SOURCES = ["paper_1905_03748_gb300/csrc/backward.cu", "paper_1905_03748_gb300/csrc/ray.cuh",
               "paper_1905_03748_gb300/csrc/quad.cuh"]
@@ -313,7 +315,7 @@ def run_ours(args):
            "samples_per_ax": samples,
            "kernel_ms": {"forward": fwd_avg, "backproject_matched": bp_avg},
            "resid_last": float(hist[-1]) if len(hist) else None,
-           "roofline": {"kernel": "fwd_quad_kernel", "bound": "l1", "achieved": l1_achieved,
+           "roofline": {"kernel": "fwd_cols_kernel", "bound": "l1", "achieved": l1_achieved,
                         "peak": l1_peak, "unit": "TB/s", "frac": l1_achieved / l1_peak,
                         "traffic": traffic,
                         "per_unit": f"{L1_BYTES_PER_SAMPLE} B gathered per quadrature sample "

@@ -326,7 +326,8 @@ TIGRE_API tigre_status tigre_cgls_end(tigre_cgls_t state);
  *        interpolated projector and the automatic forward path; bp_weight
  *        MATCHED or FDK.  Workspaces (owned by the batch, stream-ordered on
  *        opts->cuda_stream): per member 4 iterate vectors, a quad copy of the
- *        zero-bordered volume per layout and one of the padded projections
+ *        zero-bordered volume (one per layout where the automatic path takes
+ *        the quad gather kernel) and one of the padded projections
  *        (16 bytes of FP32 coefficients per padded voxel or pixel).  Otherwise as tigre_cgls_begin; TIGRE_ERR_UNSUPPORTED for
  *        other flags, projectors or weights.
  * iterate: enqueues n_iter iterations of every member (no host sync).
@@ -423,15 +424,18 @@ TIGRE_API tigre_status tigre_geometry_set_projector(tigre_geometry_t geo, int pr
  * each z-slab (0 = default 512).  Rays resident on the GPU at one time then
  * read one brick's planes, which stay in L2; at 3072^2 a single quad plane
  * of the slab is larger than L2.  In-core projections on the automatic path
- * (forward path 0, F32 volume and projections) march the same bricks when
- * the volume is wider than one brick (1024^3 x 720: 11 % faster).  Only the
- * partial sums' order changes. */
+ * (F32 volume and projections) that take the quad gather kernel march the
+ * same bricks when the volume is wider than one brick; the column kernel has
+ * no bricks.  Only the partial sums' order changes. */
 TIGRE_API tigre_status tigre_geometry_set_brick(tigre_geometry_t geo, int64_t edge);
 
 /* Kernel choice for this handle's Sec. 2.1 projector (no counterpart in the
- * paper): 0 = automatic (the quad
- * gather kernel; with 2 angles per warp when the rays of one pixel at paired
- * angles stay within 16 voxels of each other, e.g. 512^3 x 360), 1 = scalar
+ * paper): 0 = automatic (the column
+ * kernel, whose warps are detector rows and which reads one set of quads with
+ * z fastest, for calls of at least three angles and 250,000 rays on detectors
+ * of at least 16 rows that lie at most 1.9 planes apart at the axis; otherwise
+ * the quad gather kernel, with 2 angles per warp when the rays of one pixel at
+ * paired angles stay within 16 voxels of each other), 1 = scalar
  * L1 gather kernel, 2 = shared-memory slab kernel (TMA-staged; only for
  * geometries whose ray bundles fit its staging box, otherwise it reports
  * error bit 2 and NaN), 3 = quad gather kernel (two 16-byte loads per sample

@@ -187,10 +187,12 @@ struct tigre_geometry {
     int auto_angle_group = 1;
     tigre::DeviceBuffer vol_xy;       // padded volume, x fastest
     tigre::DeviceBuffer vol_yx;       // padded volume, y fastest
-    tigre::DeviceBuffer vol_qxy;      // quad volumes of the two padded layouts
+    tigre::DeviceBuffer vol_qxy;      // quad volumes of the two padded layouts (the column
+                                      // projector keeps its one set in vol_qxy)
     tigre::DeviceBuffer vol_qyx;
     tigre::DeviceBuffer proj_pad;     // zero-bordered projections for the backprojector
-    tigre::DeviceBuffer adj_xy;       // FP32 padded accumulators of the exact adjoint
+    tigre::DeviceBuffer adj_xy;       // FP32 padded accumulators of the exact adjoint (the
+                                      // column scatter keeps its quads in adj_xy)
     tigre::DeviceBuffer adj_yx;
     tigre::DeviceBuffer scratch_vol;  // FP32 volume-sized scratch
     tigre::DeviceBuffer scratch_red;  // reduction partials / device scalars

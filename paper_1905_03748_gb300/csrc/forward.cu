@@ -7,7 +7,12 @@
 // steps over the part of the ray inside the interpolant's support [-1, n],
 // K = ceil(len / (accuracy * min d)), h = len / K.
 //
-// GB300 design:
+// Whole volumes are projected by the column kernel (forward_cols.cu) where its
+// rule allows (takes_columns); this file holds that choice and the other
+// kernels: few rays, few or widely spaced detector rows, slabs of a volume, and
+// the paths a caller selects.
+//
+// GB300 design of the row-warp kernels:
 //  * The volume is copied once per call into two zero-padded layouts (x
 //    fastest, and y fastest).  Each angle reads the layout whose fastest axis
 //    is closest to e_u, so the 32 rays of a warp (adjacent pixels of one

@@ -57,7 +57,8 @@ class Result:
 def footprint_bytes(geo: dict, n_angles: int, elem: int = 4) -> int:
     """HBM one member of a batched CGLS keeps resident: x, p, s
     (volume-sized) and b, r, q (projection-sized) in elem-byte values; the
-    forward projector's quads of the two zero-bordered layouts and the
+    forward projector's quads of two zero-bordered layouts (an upper bound:
+    the column projector reads one) and the
     backprojector's quads of the zero-bordered projections (two border
     columns a side, and the rows the volume's shadow reaches beyond the
     detector, taken as 10 % + 8), four FP32 coefficients (16 bytes) per
