@@ -196,7 +196,7 @@ __device__ __forceinline__ float ld(const T* p)
 }
 
 // Trilinear sample k of ray R from the padded volume.
-template <typename TV>
+template <typename TV, bool LAYOUT1>
 __device__ __forceinline__ float tri_sample(const TV* __restrict__ vol, const Ray& R, float kf,
                                             int PF, int PFM)
 {
@@ -210,8 +210,8 @@ __device__ __forceinline__ float tri_sample(const TV* __restrict__ vol, const Ra
     const float v010 = ld(b + PF), v110 = ld(b + PF + 1);
     const float v001 = ld(b + PFM), v101 = ld(b + PFM + 1);
     const float v011 = ld(b + PFM + PF), v111 = ld(b + PFM + PF + 1);
-    const float c0 = bilinear_fm(R.layout, v000, v100, v010, v110, af, am);
-    const float c1 = bilinear_fm(R.layout, v001, v101, v011, v111, af, am);
+    const float c0 = bilinear_fm<LAYOUT1>(v000, v100, v010, v110, af, am);
+    const float c1 = bilinear_fm<LAYOUT1>(v001, v101, v011, v111, af, am);
     return fmaf(as, c1 - c0, c0);
 }
 
@@ -273,18 +273,26 @@ __global__ void __launch_bounds__(256) fwd_l1_kernel(const TV* __restrict__ vxy,
             // tiny) skips the march; the tail loop below does the work.
             const float ns = (Y1 - Y0) / D;
             const int nslab = ns < (float)(2 * kmax + 64) ? (int)ns + 1 : 0;
-            for (int j = 1; j <= nslab; ++j) {
-                const float bound = fmaf((float)j, D, Y0);
-                if (k < R.K && fmaf(kf, dy, y0) < bound) {
-                    acc += tri_sample(vol, R, kf, PF, PFM);
-                    ++k;
-                    kf += 1.0f;
+            auto march = [&](auto layout1) {
+                for (int j = 1; j <= nslab; ++j) {
+                    const float bound = fmaf((float)j, D, Y0);
+                    if (k < R.K && fmaf(kf, dy, y0) < bound) {
+                        acc += tri_sample<TV, decltype(layout1)::value>(vol, R, kf, PF, PFM);
+                        ++k;
+                        kf += 1.0f;
+                    }
                 }
-            }
+            };
+            if (layout)
+                march(std::true_type{});
+            else
+                march(std::false_type{});
         }
         // Samples not consumed above (mixed directions, or rounding at a slab
         // edge) finish in order here.
-        for (; active && k < R.K; ++k, kf += 1.0f) acc += tri_sample(vol, R, kf, PF, PFM);
+        for (; active && k < R.K; ++k, kf += 1.0f)
+            acc += layout ? tri_sample<TV, true>(vol, R, kf, PF, PFM)
+                          : tri_sample<TV, false>(vol, R, kf, PF, PFM);
     }
     if (!inside) return;
     const float out = !R.ok ? __int_as_float(0x7fc00000)  // NaN: ray failed the bounds proof
@@ -310,11 +318,16 @@ __device__ __forceinline__ float4 load_fquad(const float4* p) { return load_quad
 // outside), element (s, m, f) = (P(s,m,f), P(s,m,f+1), P(s,m+1,f),
 // P(s,m+1,f+1)).  A block makes a 32 x 32 tile of one plane from a 33 x 33
 // tile of P staged in shared memory, read along x (coalesced) in either
-// layout; blockIdx = (f tile, m tile, s).
+// layout; blockIdx = (f tile, m tile, s).  m_first: the cell is interpolated
+// along m first, which is x in layout 1.  Slabs, whose sums equal the whole
+// volume's only up to FP32 order, take f first in both layouts, so their
+// kernels hold one march per direction (two more: 512^3 x 180 in 128-plane
+// slabs 65.4 -> 69.6 ms).
 template <typename T>
 __global__ void __launch_bounds__(256) quad_from_vol_kernel(const T* __restrict__ vol,
                                                             typename QuadOf<T>::type* __restrict__ out,
-                                                            int nx, int ny, int nz, int layout)
+                                                            int nx, int ny, int nz, int layout,
+                                                            int m_first)
 {
     __shared__ T tile[33][33];
     const int PF = (layout ? ny : nx) + 2 * kPad, PM = (layout ? nx : ny) + 2 * kPad;
@@ -347,20 +360,21 @@ __global__ void __launch_bounds__(256) quad_from_vol_kernel(const T* __restrict_
         const T a = tile[i][threadIdx.x], b = tile[i][threadIdx.x + 1];
         const T c = tile[i + 1][threadIdx.x], d = tile[i + 1][threadIdx.x + 1];
         typename QuadOf<T>::type* o = out + ((int64_t)s * PM + m) * PF + f;
-        *o = layout ? bilinear_coefficients(to_f32<T>(a), to_f32<T>(c), to_f32<T>(b), to_f32<T>(d))
-                    : bilinear_coefficients(to_f32<T>(a), to_f32<T>(b), to_f32<T>(c), to_f32<T>(d));
+        *o = m_first ? bilinear_coefficients(to_f32<T>(a), to_f32<T>(c), to_f32<T>(b), to_f32<T>(d))
+                     : bilinear_coefficients(to_f32<T>(a), to_f32<T>(b), to_f32<T>(c), to_f32<T>(d));
     }
 }
 
 template <typename T>
 tigre_status build_quads(const tigre_geometry_desc& d, const T* vol, typename QuadOf<T>::type* out,
-                         int layout, cudaStream_t st)
+                         int layout, cudaStream_t st, bool slab = false)
 {
     const int nx = (int)d.n_voxel[0], ny = (int)d.n_voxel[1], nz = (int)d.n_voxel[2];
     const int PF = (layout ? ny : nx) + 2 * kPad, PM = (layout ? nx : ny) + 2 * kPad;
     if (nz + 2 * kPad > 65535) return fail(TIGRE_ERR_UNSUPPORTED, "volume too deep for one launch");
     dim3 grid((unsigned)((PF + 31) / 32), (unsigned)((PM + 31) / 32), (unsigned)(nz + 2 * kPad));
-    quad_from_vol_kernel<T><<<grid, dim3(32, 8), 0, st>>>(vol, out, nx, ny, nz, layout);
+    quad_from_vol_kernel<T><<<grid, dim3(32, 8), 0, st>>>(vol, out, nx, ny, nz, layout,
+                                                             layout && !slab);
     TIGRE_LAUNCHED("quad_from_vol_kernel");
     return TIGRE_OK;
 }
@@ -400,7 +414,8 @@ __device__ __forceinline__ float tri_sample_quad(const typename QuadOf<TV>::type
 template <typename TV>
 __device__ __forceinline__ void tri_pair_quad(const typename QuadOf<TV>::type* __restrict__ qv,
                                               const Ray& R, float kf, float ym0, float ym1, int PF,
-                                              int PFM, uint32_t bias, bool t0, bool t1, float& acc)
+                                              int PFM, uint32_t bias, bool t0, bool t1, bool m_first,
+                                              float& acc)
 {
     using Q = typename QuadOf<TV>::type;
     uint32_t f0, m0, z0, f1, m1, z1;
@@ -419,12 +434,12 @@ __device__ __forceinline__ void tri_pair_quad(const typename QuadOf<TV>::type* _
     const float4 lo1 = load_fquad(b1);
     const float4 hi1 = load_fquad(b1 + PFM);
     {
-        const float ax = R.layout ? am0 : af0, ay = R.layout ? af0 : am0;
+        const float ax = m_first ? am0 : af0, ay = m_first ? af0 : am0;
         const float c0 = bilinear_value(lo0, ax, ay), c1 = bilinear_value(hi0, ax, ay);
         if (t0) acc += fmaf(as0, c1 - c0, c0);
     }
     {
-        const float ax = R.layout ? am1 : af1, ay = R.layout ? af1 : am1;
+        const float ax = m_first ? am1 : af1, ay = m_first ? af1 : am1;
         const float c0 = bilinear_value(lo1, ax, ay), c1 = bilinear_value(hi1, ax, ay);
         if (t1) acc += fmaf(as1, c1 - c0, c0);
     }
@@ -608,7 +623,8 @@ __global__ void __launch_bounds__(256, 6) fwd_quad_kernel(
                     const bool t0 = kf < kef && sgn * ym0 < bound;
                     const bool t1 = t0 && kf + 1.0f < kef && sgn * ym1 < bound;
                     if (__any_sync(full, t0))
-                        tri_pair_quad<TV>(vol, R, kf, ym0, ym1, PF, PFM, bias, t0, t1, acc);
+                        tri_pair_quad<TV>(vol, R, kf, ym0, ym1, PF, PFM, bias, t0, t1,
+                                          !SLAB && layout, acc);
                     kf += (float)((int)t0 + (int)t1);
                 }
             } else {
@@ -630,13 +646,13 @@ __global__ void __launch_bounds__(256, 6) fwd_quad_kernel(
                     }
                 };
                 if (sgn > 0.0f) {
-                    if (layout)
-                        march(std::false_type{}, std::true_type{});
+                    if (!SLAB && layout)
+                        march(std::false_type{}, std::bool_constant<!SLAB>{});
                     else
                         march(std::false_type{}, std::false_type{});
                 } else {
-                    if (layout)
-                        march(std::true_type{}, std::true_type{});
+                    if (!SLAB && layout)
+                        march(std::true_type{}, std::bool_constant<!SLAB>{});
                     else
                         march(std::true_type{}, std::false_type{});
                 }
@@ -644,7 +660,7 @@ __global__ void __launch_bounds__(256, 6) fwd_quad_kernel(
         }
         for (; active && kf < kef; kf += 1.0f) {
             const float ym = fmaf(kf, R.d[1], R.x0[1]);
-            acc += layout ? tri_sample_quad<TV, true>(vol, R, kf, ym, PF, PFM, bias)
+            acc += !SLAB && layout ? tri_sample_quad<TV, true>(vol, R, kf, ym, PF, PFM, bias)
                           : tri_sample_quad<TV, false>(vol, R, kf, ym, PF, PFM, bias);
         }
     }
@@ -743,7 +759,7 @@ tigre_status fill_padded(const tigre_geometry_desc& d, const TV* vol, TV* out, i
 tigre_status build_quads_f32(const tigre_geometry_desc& d, const float* vol, float4* out, int layout,
                              cudaStream_t st)
 {
-    return build_quads<float>(d, vol, out, layout, st);
+    return build_quads<float>(d, vol, out, layout, st, true);
 }
 
 
@@ -960,7 +976,8 @@ tigre_status forward_impl(tigre_geometry* g, const void* vol, tigre_dtype vt, vo
         for (int l = 0; l < 2; ++l) {
             if (!need[l]) continue;
             if (use_quad)
-                TIGRE_TRY(build_quads<TV>(d, (const TV*)vol, (Q*)qbufs[l]->ptr, l, st));
+                TIGRE_TRY(build_quads<TV>(d, (const TV*)vol, (Q*)qbufs[l]->ptr, l, st,
+                                          in_core_bricks(g, vt) && pt == TIGRE_F32));
             else
                 TIGRE_TRY(fill_padded<TV>(d, (const TV*)vol, (TV*)bufs[l]->ptr, l, st));
         }

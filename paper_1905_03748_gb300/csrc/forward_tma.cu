@@ -281,7 +281,8 @@ __global__ void __launch_bounds__(256) fwd_tma_kernel(const __grid_constant__ CU
             if (!ok && n > 0) bad = true;
             if (!ok && tid == 0) atomicOr(err, kErrTile);
             float kf = (float)k0;
-            for (int j = 0; j < nmax; ++j, kf += 1.0f) {
+            auto samples = [&](auto layout1) {
+                for (int j = 0; j < nmax; ++j, kf += 1.0f) {
                 if (ok && j < n) {
                     int i_f, i_m, i_s;
                     float af, am, as;
@@ -294,11 +295,16 @@ __global__ void __launch_bounds__(256) fwd_tma_kernel(const __grid_constant__ CU
                     const float v001 = to_f32<TV>(b[C::SP]), v101 = to_f32<TV>(b[C::SP + 1]);
                     const float v011 = to_f32<TV>(b[C::SP + C::FB]);
                     const float v111 = to_f32<TV>(b[C::SP + C::FB + 1]);
-                    const float c0 = bilinear_fm(P->layout, v000, v100, v010, v110, af, am);
-                    const float c1 = bilinear_fm(P->layout, v001, v101, v011, v111, af, am);
+                    const float c0 = bilinear_fm<decltype(layout1)::value>(v000, v100, v010, v110, af, am);
+                    const float c1 = bilinear_fm<decltype(layout1)::value>(v001, v101, v011, v111, af, am);
                     acc += fmaf(as, c1 - c0, c0);
                 }
             }
+            };
+            if (P->layout)
+                samples(std::true_type{});
+            else
+                samples(std::false_type{});
             __syncthreads();  // every warp is done with this stage
             int k3 = k2;
             if (s + 2 < nslab) {

@@ -64,11 +64,12 @@ __device__ __forceinline__ float bilinear_value(const float4& e, float fx, float
 
 // The same from the taps of a cell on a layout's (f, m) axes: x is f in
 // layout 0 and m in layout 1.
-__device__ __forceinline__ float bilinear_fm(int layout, float v00, float vf, float vm, float vfm,
-                                             float af, float am)
+template <bool LAYOUT1>
+__device__ __forceinline__ float bilinear_fm(float v00, float vf, float vm, float vfm, float af,
+                                             float am)
 {
-    return layout ? bilinear_value(bilinear_coefficients(v00, vm, vf, vfm), am, af)
-                  : bilinear_value(bilinear_coefficients(v00, vf, vm, vfm), af, am);
+    return LAYOUT1 ? bilinear_value(bilinear_coefficients(v00, vm, vf, vfm), am, af)
+                   : bilinear_value(bilinear_coefficients(v00, vf, vm, vfm), af, am);
 }
 
 // The same split with the integer part left biased: b = i + 0x4B000000, the
