@@ -22,6 +22,7 @@ namespace tigre {
 namespace {
 
 constexpr double kPi = 3.14159265358979323846;
+constexpr int kFdkMaxRowBytes = 160 * 1024;  // the longest detector row
 
 // One block per (row q, angle a): out[a][q][p] = wa * sum_k w(k) y[k] h(p-k).
 // The kernel is even and vanishes at even non-zero offsets, so each output
@@ -178,7 +179,7 @@ tigre_status fdk_impl(tigre_geometry* g, const void* proj, tigre_dtype pt, void*
     const tigre_geometry_desc& d = g->desc;
     const int nu = (int)d.n_det[0], nv = (int)d.n_det[1];
     const int64_t na = (int64_t)g->angles.size();
-    if ((size_t)nu * sizeof(float) > 160 * 1024)
+    if ((size_t)nu * sizeof(float) > (size_t)kFdkMaxRowBytes)
         return fail(TIGRE_ERR_UNSUPPORTED, "detector rows longer than 40960 pixels");
     if (nv > 2147483647 || na > 65535) return fail(TIGRE_ERR_UNSUPPORTED, "too many rows or angles");
     // Ram-Lak taps at odd offsets and the angular factors (FP64 on the host).
@@ -208,25 +209,28 @@ tigre_status fdk_impl(tigre_geometry* g, const void* proj, tigre_dtype pt, void*
         status = dispatch_dtype(pt, [&](auto tag) -> tigre_status {
             using TP = decltype(tag);
             // Blocks of 8 rows up to 2048 columns (73 KB: three per SM), of 4
-            // up to 8192 (164 KB); longer rows one by one.
-            auto rows = [&](auto kern, int R) -> tigre_status {
-                const int H = ((nu + 1) / 2 + 3) & ~3;
-                const int bytes = (int)sizeof(float) * (2 * R * H + 2 * H + 4);
-                if (bytes > 48 * 1024)
-                    TIGRE_CUDA(cudaFuncSetAttribute(
-                        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-                kern<<<dim3((unsigned)((nv + R - 1) / R), (unsigned)na), kFdkThreads, bytes, st>>>(
+            // up to 8192 (164 KB); longer rows one by one.  An instance's
+            // shared-memory limit is the process's: every call sets it to what
+            // the instance's longest rows need, never to its own rows' bytes,
+            // which another thread's launch may exceed.
+            auto rows = [&](auto kern, int R, int nu_max) -> tigre_status {
+                const auto bytes = [R](int n) {
+                    const int H = ((n + 1) / 2 + 3) & ~3;
+                    return (int)sizeof(float) * (2 * R * H + 2 * H + 4);
+                };
+                TIGRE_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                bytes(nu_max)));
+                kern<<<dim3((unsigned)((nv + R - 1) / R), (unsigned)na), kFdkThreads, bytes(nu), st>>>(
                     (const TP*)proj, filt, dtab, dtab + (nu / 2 + 1), nu, nv, h0, u0,
                     (float)d.d_det[0], v0, (float)d.d_det[1], (float)(d.DSD * d.DSD));
                 TIGRE_LAUNCHED("fdk_filter_rows_kernel");
                 return TIGRE_OK;
             };
-            if (nu <= 2048) return rows(fdk_filter_rows_kernel<TP, 8>, 8);
-            if (nu <= 8192) return rows(fdk_filter_rows_kernel<TP, 4>, 4);
-            if (smem > 48 * 1024)
-                TIGRE_CUDA(cudaFuncSetAttribute(fdk_filter_kernel<TP>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)smem));
+            if (nu <= 2048) return rows(fdk_filter_rows_kernel<TP, 8>, 8, 2048);
+            if (nu <= 8192) return rows(fdk_filter_rows_kernel<TP, 4>, 4, 8192);
+            TIGRE_CUDA(cudaFuncSetAttribute(fdk_filter_kernel<TP>,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            kFdkMaxRowBytes));
             fdk_filter_kernel<TP><<<dim3((unsigned)nv, (unsigned)na), 256, smem, st>>>(
                 (const TP*)proj, filt, dtab, dtab + (nu / 2 + 1), nu, nv, h0, u0,
                 (float)d.d_det[0], v0, (float)d.d_det[1], (float)(d.DSD * d.DSD));
