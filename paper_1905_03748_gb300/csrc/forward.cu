@@ -801,18 +801,6 @@ static void needed_layouts(const tigre_geometry* g, int64_t a0, int64_t na, bool
 
 static tigre_status brick_pixel_ranges(tigre_geometry* g, const int2** out);
 
-// Whether an in-core projection marches x-y bricks: the automatic path, F32
-// volume, projector interpolated, and a volume wider than one brick.  Its
-// rays then read one brick's planes at a time, which stay in L2 (1024^3 x
-// 720: 1790 vs 2012 ms of kernels); a 512^2 plane is one brick.
-static bool in_core_bricks(const tigre_geometry* g, tigre_dtype vt)
-{
-    const tigre_geometry_desc& d = g->desc;
-    const int64_t e = g->brick;
-    return g->fwd_path == 0 && vt == TIGRE_F32 && g->projector == TIGRE_PROJ_INTERPOLATED &&
-           e > 0 && (d.n_voxel[0] > e || d.n_voxel[1] > e);
-}
-
 // Whether a projection of na angles takes the column projector
 // (forward_cols.cu): the automatic path with the interpolated projector, where
 // its 8-row warps are full and read near planes, and there are enough of
@@ -842,9 +830,29 @@ static bool takes_columns(const tigre_geometry* g, int64_t na)
     return g->fwd_path == 0 && g->projector == TIGRE_PROJ_INTERPOLATED && column_warps_pay(g, na);
 }
 
-// Its launch over the angles [a0, a0 + na): blocks of four neighbouring angles
-// (the groups of the four-angle quad kernel), or of one where there are few
-// (the groups would leave warps empty).
+// Whether an in-core projection marches x-y bricks: the automatic path, F32
+// volume, projector interpolated, a volume wider than one brick, and angles
+// too few or rows too few for the column projector even over the full range.
+// A ray then reads one brick's planes at a time, which stay in L2 (1024^2 x
+// 64, 180 angles of 24 rows 3.1 planes apart: 14.3 ms against 16.5 without
+// bricks); a 512^2 plane is one brick.  The full range decides for every
+// range, because bricks add their partial sums and no other path does: a
+// range equals the full projection's slice bit for bit.  (One or two angles
+// of a volume whose full range takes columns are faster without bricks:
+// 1024^3 one angle 9.05 -> 8.59 ms, two 11.8 -> 12.0; 640 x 600 x 512 2.63 ->
+// 2.10, 3.00 -> 2.80.)
+static bool in_core_bricks(const tigre_geometry* g, tigre_dtype vt)
+{
+    const tigre_geometry_desc& d = g->desc;
+    const int64_t e = g->brick;
+    return g->fwd_path == 0 && vt == TIGRE_F32 && g->projector == TIGRE_PROJ_INTERPOLATED &&
+           e > 0 && (d.n_voxel[0] > e || d.n_voxel[1] > e) &&
+           !takes_columns(g, (int64_t)g->angles.size());
+}
+
+// Launch of the column projector over the angles [a0, a0 + na): blocks of four
+// neighbouring angles (the groups of the four-angle quad kernel), or of one
+// where there are few (the groups would leave warps empty).
 constexpr int64_t kColsGroupAngles = 8;
 
 template <typename TP>
