@@ -286,11 +286,16 @@ tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* 
                                     int64_t vol_stride, int64_t proj_stride, cudaStream_t st)
 {
     const FwdConst c = make_fwd_const(g);
-    // Warps of 8 detector rows x 8 columns, or 16 x 4 where one plane of quads
-    // is larger than 6.5 MB: fewer strips of planes live in L2 at a time
-    // (1024^3 x 180: 426 ms against 459, 768^3 x 180: 176 / 182; 512^3 x 360:
-    // 94.5 / 93.3, 128^3 x 90: 0.519 / 0.495).
-    const int rows = (int64_t)c.nx * c.ny >= 640 * 640 ? 16 : 8;
+    // Warps of 8 detector rows x 8 columns, or 16 x 4 on planes of quads larger
+    // than 6.5 MB, where fewer strips of planes then live in L2 at a time, if the
+    // detector is tall (16-row / 8-row ms, 60 angles of 256 rows: 640^2 13.8 /
+    // 14.1, 1024^2 39.4 / 40.4; of 1024 rows: 1024^2 160 / 180) or one such warp
+    // holds all its rows (640^2 x 16, 180 angles: 3.15 / 3.44).  Between the two
+    // the taller tile costs more than it saves (180 angles: 1024^2 of 24 rows 18.6
+    // / 14.1, 64 rows 33.9 / 31.2, 192 rows 80.8 / 79.0), and on small planes always
+    // (512^3 x 360: 94.5 / 93.3, 128^3 x 90: 0.519 / 0.495).
+    const bool large = (int64_t)c.nx * c.ny >= 640 * 640;
+    const int rows = large && (c.nv >= 224 || c.nv <= 16) ? 16 : 8;
     const int cols = 2 * (32 / rows) * (kColWarps / ag), tiles = (c.nv + rows - 1) / rows;
     dim3 grid((unsigned)((c.nu + cols - 1) / cols), (unsigned)groups, (unsigned)(tiles * batch));
     ColGeom w;
