@@ -801,10 +801,9 @@ static void needed_layouts(const tigre_geometry* g, int64_t a0, int64_t na, bool
 
 static tigre_status brick_pixel_ranges(tigre_geometry* g, const int2** out);
 
-// Whether a projection of na angles takes the column projector
-// (forward_cols.cu): the automatic path with the interpolated projector, where
-// its 8-row warps are full and read near planes, and there are enough of
-// them.  Both sides measured (column / quad kernel, ms):
+// Whether warps of detector rows suit na angles: 8-row warps are full and read
+// near planes, and there are enough of them.  Both sides measured (forward
+// projection, column / quad kernel, ms):
 //   rows fill the warps: 512^2 x 16 volume, 180 angles: 16 rows 2.13 / 2.17,
 //     24 rows 2.86 / 3.11; 512^2 x 12, 12 rows 1.96 / 1.68; 9 rows 1.53 / 1.34;
 //   neighbouring rows at most 1.9 planes apart at the axis: 512^2 x 64, 180
@@ -825,9 +824,81 @@ bool column_warps_pay(const tigre_geometry* g, int64_t na)
            na >= kColsMinAngles && d.n_det[0] * nv * na >= kColsMinRays;
 }
 
-static bool takes_columns(const tigre_geometry* g, int64_t na)
+// What the forward projector asks for besides, of the rows and columns that the
+// volume's shadow covers at the axis (its height; the mean width of its x-y
+// rectangle, perimeter / pi).  Both sides measured:
+//   * Their rows fill 8-row warps where the detector is taller than the shadow.
+//     180 angles, quad / column time: 20 rows of 400 (four tiles) 0.82, 24 of 400
+//     (four) 0.87 to 0.95, 24 of 200 (three) 0.92 to 1.07.
+//   * Enough of the rays cross the volume (quad / column time: 15,000 to 61,000
+//     0.71 to 0.93, 133,000 to 282,000 1.17 to 1.19 and 0.77).
+//   * Rows times angles times columns per voxel, from planes of 128^2 on: few
+//     rays share few cells.  Quad / column time, BF16, 0.87 columns a voxel, 12,
+//     24, 48 and 96 angles round the circle: 512^2 of 24 rows -, 0.68, 0.96, 1.06;
+//     40 rows -, 0.79, 1.06, 1.14; 128 rows 1.02, 1.08, 1.31, 1.42; 1024^2 of 64
+//     rows 0.76, 0.84, 1.02, 1.14; 1.74 columns a voxel, 64 rows 0.93, 0.94, 1.07,
+//     1.10 (half a degree apart 1.06, 1.11, 1.14, 1.14).  Fewer columns count as
+//     0.87 a voxel: they cost the quad kernel more (544 x 857 x 45 under 40 x 233,
+//     204 angles 2.98 / 6.25 ms).  Planes under 512^2 are level at few angles from
+//     80 rows on, all planes from 256; and one set of quads to build instead of
+//     two decides where the rays take few samples per voxel (529 x 424 x 159
+//     under 256 x 39, 26 angles, 5.2 samples 0.65 / 0.99 ms).
+//   * More rows on large planes, where the 2-angle quad kernel and F32 bricks
+//     gain (column / quad ms): 640^2 of 24 rows, 720 angles 16.7 / 15.6 (BF16);
+//     1024^2 of 40 rows, 720 angles 78.9 / 68.7 (F32) and 75.7 (BF16), of 64 rows,
+//     180 angles 30.8 / 33.2 and 34.7.  One tile of 16 rows pays up to 896^2
+//     (640^2, 180 angles 3.15 / 3.40, BF16).
+constexpr double kColsMinCrossing = 120000.0, kColsMinRowAngles = 2440.0, kColsMinDensity = 0.87;
+constexpr double kColsRowsSmall = 80.0, kColsRowsAny = 256.0;  // rows that pay at any angles
+constexpr double kColsRows640 = 48.0, kColsRows896 = 64.0;     // least rows on such planes
+constexpr double kColsBuildSamples = 5.6;                      // samples per voxel
+
+static bool columns_pay(const tigre_geometry* g, int64_t a0, int64_t na)
 {
-    return g->fwd_path == 0 && g->projector == TIGRE_PROJ_INTERPOLATED && column_warps_pay(g, na);
+    if (!column_warps_pay(g, na)) return false;
+    const tigre_geometry_desc& d = g->desc;
+    const double pi = 3.14159265358979323846, mag = d.DSD / d.DSO, nv = (double)d.n_det[1];
+    const double height = (double)d.n_voxel[2] * d.d_voxel[2] * mag / d.d_det[1];
+    const double centre = 0.5 * nv + (d.off_origin[2] * mag - d.off_det[1]) / d.d_det[1];
+    const double lo = std::max(0.0, centre - 0.5 * height), hi = std::min(nv, centre + 0.5 * height);
+    const bool fills = hi - lo >= 0.8 * nv;  // the near side's shadow is taller
+    const double rows = fills ? nv : hi - lo;
+    if (!fills && 4.0 * rows <= 24.0 * (std::ceil(hi / 8.0) - std::floor(lo / 8.0))) return false;
+    const double lx = (double)d.n_voxel[0] * d.d_voxel[0], ly = (double)d.n_voxel[1] * d.d_voxel[1];
+    const double width = 2.0 * (lx + ly) / pi, chord = lx * ly / width;
+    const double rays = (double)na * (hi - lo) *
+                        std::min((double)d.n_det[0], width * mag / d.d_det[0]);
+    if (rays < kColsMinCrossing) return false;
+    const int64_t plane = d.n_voxel[0] * d.n_voxel[1];
+    const double voxel = std::min(d.d_voxel[0], d.d_voxel[1]);
+    if (plane >= 128 * 128 && rows < (plane < 512 * 512 ? kColsRowsSmall : kColsRowsAny) &&
+        rows * (double)na * std::max(kColsMinDensity, voxel * mag / d.d_det[0]) < kColsMinRowAngles) {
+        bool need[2];
+        needed_layouts(g, a0, na, need);
+        const double step = d.accuracy * std::min(voxel, d.d_voxel[2]);
+        if (!need[0] || !need[1] ||
+            rays * chord / step > kColsBuildSamples * (double)padded_elems(d))
+            return false;
+    }
+    if (plane >= 896 * 896) return rows >= kColsRows896;
+    return plane < 640 * 640 || rows >= kColsRows640 || d.n_det[1] == 16;
+}
+
+// Volumes wider than one x-y brick (the in-core ones march them on the quad
+// path, which changes the sums' last bits).
+static bool wider_than_a_brick(const tigre_geometry* g)
+{
+    return g->brick > 0 && (g->desc.n_voxel[0] > g->brick || g->desc.n_voxel[1] > g->brick);
+}
+
+// Whether the projection of [a0, a0 + na) takes the column projector
+// (forward_cols.cu).  A range of a wide volume takes it only if the full range
+// does, which then marches no bricks: every range is the full projection's
+// slice bit for bit.
+static bool takes_columns(const tigre_geometry* g, int64_t a0, int64_t na)
+{
+    return g->fwd_path == 0 && g->projector == TIGRE_PROJ_INTERPOLATED && columns_pay(g, a0, na) &&
+           (!wider_than_a_brick(g) || columns_pay(g, 0, (int64_t)g->angles.size()));
 }
 
 // Whether an in-core projection marches x-y bricks: the automatic path, F32
@@ -843,11 +914,8 @@ static bool takes_columns(const tigre_geometry* g, int64_t na)
 // 2.10, 3.00 -> 2.80.)
 static bool in_core_bricks(const tigre_geometry* g, tigre_dtype vt)
 {
-    const tigre_geometry_desc& d = g->desc;
-    const int64_t e = g->brick;
     return g->fwd_path == 0 && vt == TIGRE_F32 && g->projector == TIGRE_PROJ_INTERPOLATED &&
-           e > 0 && (d.n_voxel[0] > e || d.n_voxel[1] > e) &&
-           !takes_columns(g, (int64_t)g->angles.size());
+           wider_than_a_brick(g) && !takes_columns(g, 0, (int64_t)g->angles.size());
 }
 
 // Launch of the column projector over the angles [a0, a0 + na): blocks of four
@@ -899,7 +967,7 @@ tigre_status forward_workspace(tigre_geometry* g, tigre_dtype vt, int64_t a0, in
         return tma_workspace(g, dtype_size(vt), need);
     }
     const bool use_quad = !siddon && (g->fwd_path == 0 || g->fwd_path >= 3);
-    if (takes_columns(g, na)) {
+    if (takes_columns(g, a0, na)) {
         const bool all = a0 == 0 && na == (int64_t)g->angles.size();
         if (!all && na >= kColsGroupAngles) {
             const int* table = nullptr;
@@ -970,7 +1038,7 @@ tigre_status forward_impl(tigre_geometry* g, const void* vol, tigre_dtype vt, vo
         DeviceBuffer* bufs[2] = {&g->vol_xy, &g->vol_yx};
         DeviceBuffer* qbufs[2] = {&g->vol_qxy, &g->vol_qyx};
         static_assert(sizeof(Q) == 4 * sizeof(float), "a quad is four FP32 coefficients");
-        if (takes_columns(g, na)) {
+        if (takes_columns(g, a0, na)) {
             if (d.n_voxel[2] + 2 * kPad > 65535)
                 return fail(TIGRE_ERR_UNSUPPORTED, "volume too deep for one launch");
             float4* quads = (float4*)g->vol_qxy.ptr;
@@ -1065,7 +1133,7 @@ tigre_status forward_impl(tigre_geometry* g, const void* vol, tigre_dtype vt, vo
 
 void batch_quad_layouts(const tigre_geometry* g, bool need[2])
 {
-    if (takes_columns(g, (int64_t)g->angles.size())) {
+    if (takes_columns(g, 0, (int64_t)g->angles.size())) {
         need[0] = true;
         need[1] = false;
         return;
@@ -1090,7 +1158,7 @@ tigre_status forward_batch_impl(tigre_geometry* g, const void* vols, void* projs
     needed_layouts(g, 0, na, need);
     const int64_t nvox = d.n_voxel[0] * d.n_voxel[1] * d.n_voxel[2];
     const int64_t pe = (int64_t)padded_elems(d);
-    const bool columns = takes_columns(g, na);
+    const bool columns = takes_columns(g, 0, na);
     if (columns && d.n_voxel[2] + 2 * kPad > 65535)
         return fail(TIGRE_ERR_UNSUPPORTED, "volume too deep for one launch");
     return dispatch_dtype(dt, [&](auto tag) -> tigre_status {

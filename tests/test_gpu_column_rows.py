@@ -18,11 +18,11 @@ def geometry(n, nu, nv):
 
 
 CASES = {  # (volume, columns, rows, angles, range)
-    "16 rows, one tile": ((656, 648, 12), 701, 16, 180, (0, 180)),
-    "16-row warps, ragged": ((644, 660, 225), 333, 233, 13, (0, 13)),
-    "16-row warps, a range": ((652, 640, 220), 301, 226, 23, (5, 13)),
-    "8-row warps, ragged": ((648, 644, 110), 459, 111, 29, (0, 29)),
-    "8-row warps, a range": ((640, 641, 200), 401, 202, 40, (7, 15)),
+    "16 rows, one tile": ((656, 648, 12), 701, 16, 230, (0, 230)),
+    "16-row warps, ragged": ((644, 660, 250), 333, 261, 13, (0, 13)),
+    "16-row warps, a range": ((652, 640, 250), 301, 258, 23, (5, 13)),
+    "8-row warps, ragged": ((648, 644, 110), 459, 111, 60, (0, 60)),
+    "8-row warps, a range": ((640, 641, 200), 401, 202, 40, (7, 33)),
 }
 
 
@@ -46,9 +46,9 @@ def test_rows_equal_the_quad_kernel(tigre, name):
 @pytest.mark.parametrize("graph", [False, True])
 def test_batched_16_row_warps(tigre, graph):
     """Members of a batch (two iterations of CGLS) equal their problems alone."""
-    geo, ang = geometry((640, 644, 225), 333, 227), synth.angles(13, first=0.2)
+    geo, ang = geometry((640, 644, 250), 333, 259), synth.angles(13, first=0.2)
     with tigre.Geometry(geo, ang) as G:
-        bs = [torch.from_numpy(np.random.default_rng(i).random((13, 227, 333)).astype(np.float32)).cuda()
+        bs = [torch.from_numpy(np.random.default_rng(i).random((13, 259, 333)).astype(np.float32)).cuda()
               for i in range(2)]
         ref = []
         for b in bs:
@@ -67,3 +67,31 @@ def test_batched_16_row_warps(tigre, graph):
     for (x, h), xb, hb in zip(ref, xs, hs):
         assert torch.equal(x, xb)
         assert np.array_equal(h, hb)
+
+
+ROUTES = {  # (volume, columns, rows, row pitch or None, angles): launches of a projection
+    "a small object under a tall detector": (((29, 194, 37), 416, 764, 1.8, 12), 3),
+    "a shadow of 20 rows over four tiles": (((200, 210, 20), 300, 400, 1.0, 150), 3),
+    "few rows at few angles": (((512, 520, 24), 512, 24, None, 24), 3),
+    "few rows at many angles": (((512, 520, 24), 512, 24, None, 200), 2),
+    "few rows of a tall volume": (((400, 410, 200), 256, 40, 0.4, 26), 2),
+    "tall detector, few angles": (((300, 310, 90), 301, 97, None, 14), 2),
+}
+
+
+@pytest.mark.parametrize("name", list(ROUTES))
+def test_calls_too_small_for_columns_take_quads(tigre, name):
+    """Where few rays cross the volume, or few rows at few angles do, the quad
+    kernel (two sets of quads and a march: three launches) is the faster one; the
+    results are the same bits."""
+    (n, nu, nv, dv, na), launches = ROUTES[name]
+    geo = geometry(n, nu, nv)
+    if dv:
+        geo["d_det"] = (560.0 / nu * n[1] / 640.0, dv * 0.4 * 1.5)
+    with tigre.Geometry(geo, synth.angles(na, first=0.1)) as G:
+        v = torch.from_numpy(synth.random_volume(G.vol_shape, seed=nu)).cuda().to(torch.bfloat16)
+        n0 = tigre.tigre_launch_count()
+        out = G.forward(v)
+        assert tigre.tigre_launch_count() - n0 == launches
+        tigre.tigre_geometry_set_forward_path(G.handle, tigre.FWD_QUAD)
+        assert torch.equal(out, G.forward(v))
