@@ -210,16 +210,18 @@ tigre_status fdk_impl(tigre_geometry* g, const void* proj, tigre_dtype pt, void*
             using TP = decltype(tag);
             // Blocks of 8 rows up to 2048 columns (73 KB: three per SM), of 4
             // up to 8192 (164 KB); longer rows one by one.  An instance's
-            // shared-memory limit is the process's: every call sets it to what
-            // the instance's longest rows need, never to its own rows' bytes,
-            // which another thread's launch may exceed.
+            // shared-memory limit is the process's: a call beyond the default
+            // 48 KB sets it to what the instance's longest rows need, never to
+            // its own rows' bytes, which another thread's launch may exceed
+            // (below 48 KB the setting would cost 1 to 2 us of a 43 us call).
             auto rows = [&](auto kern, int R, int nu_max) -> tigre_status {
                 const auto bytes = [R](int n) {
                     const int H = ((n + 1) / 2 + 3) & ~3;
                     return (int)sizeof(float) * (2 * R * H + 2 * H + 4);
                 };
-                TIGRE_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                bytes(nu_max)));
+                if (bytes(nu) > 48 * 1024)
+                    TIGRE_CUDA(cudaFuncSetAttribute(
+                        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(nu_max)));
                 kern<<<dim3((unsigned)((nv + R - 1) / R), (unsigned)na), kFdkThreads, bytes(nu), st>>>(
                     (const TP*)proj, filt, dtab, dtab + (nu / 2 + 1), nu, nv, h0, u0,
                     (float)d.d_det[0], v0, (float)d.d_det[1], (float)(d.DSD * d.DSD));
@@ -228,9 +230,10 @@ tigre_status fdk_impl(tigre_geometry* g, const void* proj, tigre_dtype pt, void*
             };
             if (nu <= 2048) return rows(fdk_filter_rows_kernel<TP, 8>, 8, 2048);
             if (nu <= 8192) return rows(fdk_filter_rows_kernel<TP, 4>, 4, 8192);
-            TIGRE_CUDA(cudaFuncSetAttribute(fdk_filter_kernel<TP>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            kFdkMaxRowBytes));
+            if (smem > 48 * 1024)
+                TIGRE_CUDA(cudaFuncSetAttribute(fdk_filter_kernel<TP>,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                kFdkMaxRowBytes));
             fdk_filter_kernel<TP><<<dim3((unsigned)nv, (unsigned)na), 256, smem, st>>>(
                 (const TP*)proj, filt, dtab, dtab + (nu / 2 + 1), nu, nv, h0, u0,
                 (float)d.d_det[0], v0, (float)d.d_det[1], (float)(d.DSD * d.DSD));
