@@ -939,12 +939,12 @@ static tigre_status run_columns(tigre_geometry* g, const float4* quads, TP* proj
             TIGRE_TRY(range_group_table(g, 1, a0, na, &table, &groups));
         }
         for (int64_t s = 0; s < groups; s += 65535)
-            TIGRE_TRY(launch_forward_columns<TP>(g, quads, proj, (int)a0, table + 4 * s, 4,
+            TIGRE_TRY(launch_forward_columns<TP>(g, quads, proj, (int)a0, table + 4 * s,
                                                  std::min<int64_t>(65535, groups - s), batch,
                                                  vol_stride, proj_stride, st));
         return TIGRE_OK;
     }
-    return launch_forward_columns<TP>(g, quads, proj, (int)a0, nullptr, 1, na, batch, vol_stride,
+    return launch_forward_columns<TP>(g, quads, proj, (int)a0, nullptr, na, batch, vol_stride,
                                       proj_stride, st);
 }
 

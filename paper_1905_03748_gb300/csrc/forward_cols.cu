@@ -39,7 +39,7 @@
 namespace tigre {
 namespace {
 
-constexpr int kColWarps = 4;   // warps per block
+constexpr int kColWarps = 4;   // warps per block, angles per group
 constexpr int kColBlocks = 9;  // blocks per SM (56 registers)
 
 // Element (y, x, s) of the column quads, s fastest: the bilinear coefficients
@@ -104,7 +104,8 @@ __device__ __forceinline__ void load_cell(const float4* __restrict__ q, uint32_t
 struct ColGeom {
     uint32_t SX, SY;  // quads between x and y neighbours
     uint32_t bias;    // of an element index built from split_bits parts
-    int ag, tiles;  // angles per block (1 or kColWarps), row tiles of one member
+    int ag;  // angles per block: 1 (at four tiles of columns) or kColWarps (at one)
+    int tiles;  // row tiles of one member
     int64_t vol_stride, proj_stride;  // between a batch's members
 };
 
@@ -282,7 +283,7 @@ tigre_status build_quad_columns(const tigre_geometry_desc& d, const T* vol, floa
 
 template <typename TP>
 tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* proj, int a_first,
-                                    const int* table, int ag, int64_t groups, int batch,
+                                    const int* table, int64_t groups, int batch,
                                     int64_t vol_stride, int64_t proj_stride, cudaStream_t st)
 {
     const FwdConst c = make_fwd_const(g);
@@ -296,6 +297,7 @@ tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* 
     // (512^3 x 360: 94.5 / 93.3, 128^3 x 90: 0.519 / 0.495).
     const bool large = (int64_t)c.nx * c.ny >= 640 * 640;
     const int rows = large && (c.nv >= 224 || c.nv <= 16) ? 16 : 8;
+    const int ag = table ? kColWarps : 1;
     const int cols = 2 * (32 / rows) * (kColWarps / ag), tiles = (c.nv + rows - 1) / rows;
     dim3 grid((unsigned)((c.nu + cols - 1) / cols), (unsigned)groups, (unsigned)(tiles * batch));
     ColGeom w;
@@ -318,8 +320,8 @@ tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* 
     template tigre_status build_quad_columns<T>(const tigre_geometry_desc&, const T*, float4*,  \
                                                 cudaStream_t);                                  \
     template tigre_status launch_forward_columns<T>(tigre_geometry*, const float4*, T*, int,    \
-                                                    const int*, int, int64_t, int, int64_t,     \
-                                                    int64_t, cudaStream_t);
+                                                    const int*, int64_t, int, int64_t, int64_t, \
+                                                    cudaStream_t);
 TIGRE_COLS(float)
 TIGRE_COLS(__nv_bfloat16)
 TIGRE_COLS(__half)

@@ -10,13 +10,13 @@ namespace tigre {
 template <typename T>
 tigre_status build_quad_columns(const tigre_geometry_desc& d, const T* vol, float4* out,
                                 cudaStream_t st);
-// Projection of `groups` groups of `ag` (1 or 2) angles: table[i * ag + j] is
-// an angle relative to a_first or -1, or with a null table (ag = 1) group i is
-// angle i.  A batch's members lie vol_stride quads and proj_stride elements
-// apart.
+// Projection of `groups` groups of four angles: table[4 i + j] is an angle
+// relative to a_first or -1; or with a null table of the `groups` angles from
+// a_first, one per block.  A batch's members lie vol_stride quads and
+// proj_stride elements apart.
 template <typename TP>
 tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* proj, int a_first,
-                                    const int* table, int ag, int64_t groups, int batch,
+                                    const int* table, int64_t groups, int batch,
                                     int64_t vol_stride, int64_t proj_stride, cudaStream_t st);
 
 // Exact transpose of the projection of the angles [a0, a0 + na) (adjoint_cols.cu)
