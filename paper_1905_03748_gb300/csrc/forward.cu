@@ -29,6 +29,7 @@
 //  * floor() without conversion instructions (split_floor).
 #include <algorithm>
 #include <cmath>
+#include <functional>
 #include <type_traits>
 #include <vector>
 
@@ -918,34 +919,60 @@ static bool in_core_bricks(const tigre_geometry* g, tigre_dtype vt)
            wider_than_a_brick(g) && !takes_columns(g, 0, (int64_t)g->angles.size());
 }
 
-// Launch of the column projector over the angles [a0, a0 + na): blocks of four
-// neighbouring angles (the groups of the four-angle quad kernel), or of one
-// where there are few (the groups would leave warps empty).
+// The angle groups of a column launch over [a0, a0 + na): four neighbouring
+// angles to a block, or one where there are few (short groups leave warps empty;
+// ms with four / one to a block at 4, 5, 7 and 9 angles: 128^3 under 256^2 0.108 /
+// 0.121, 0.146 / 0.134, 0.164 / 0.170, 0.196 / 0.193; 256^3 under 384^2 0.427 /
+// 0.428, 0.501 / 0.453, 0.595 / 0.582, 0.728 / 0.695; 512^3 1.67 / 1.87, 2.14 /
+// 2.19, 2.52 / 2.81, 3.23 / 3.41).  The full range has its table from the handle's
+// creation.  A range of sorted angles takes them as they come (as fast as its
+// table: 512^3, 60 of 360 angles 16.15 and 16.16), so it needs nothing prepared.
+// Other ranges get a table of neighbours (golden angles, 512^3, 60 of 360: 17.6
+// with, 22.1 without), made when the workspaces are, outside a stream capture;
+// without one the order costs time only.
 constexpr int64_t kColsGroupAngles = 8;
+
+static bool sorted_angles(const tigre_geometry* g, int64_t a0, int64_t na)
+{
+    const double* t = g->angles.data() + a0;
+    return std::is_sorted(t, t + na) || std::is_sorted(t, t + na, std::greater<double>());
+}
+
+static bool columns_want_table(const tigre_geometry* g, int64_t a0, int64_t na)
+{
+    const bool all = a0 == 0 && na == (int64_t)g->angles.size();
+    return !all && na >= kColsGroupAngles && !sorted_angles(g, a0, na);
+}
+
+static ColGroups column_groups(const tigre_geometry* g, int64_t a0, int64_t na)
+{
+    if (na < kColsGroupAngles) return {false, nullptr, na};
+    if (a0 == 0 && na == (int64_t)g->angles.size())
+        return {true, (const int*)g->angle_groups[1].ptr, g->n_groups[1]};
+    const std::pair<int64_t, int64_t> key(a0, na);
+    const auto it = g->range_groups[1].find(key);
+    if (it != g->range_groups[1].end())
+        return {true, (const int*)it->second.ptr, g->range_n_groups[1].at(key)};
+    return {true, nullptr, (na + 3) / 4};
+}
 
 template <typename TP>
 static tigre_status run_columns(tigre_geometry* g, const float4* quads, TP* proj, int64_t a0,
                                 int64_t na, int batch, int64_t vol_stride, int64_t proj_stride,
                                 cudaStream_t st)
 {
-    const bool all = a0 == 0 && na == (int64_t)g->angles.size();
-    const int* table = nullptr;
-    int64_t groups = 0;
-    if (na >= kColsGroupAngles) {
-        if (all) {
-            table = (const int*)g->angle_groups[1].ptr;
-            groups = g->n_groups[1];
-        } else {
-            TIGRE_TRY(range_group_table(g, 1, a0, na, &table, &groups));
-        }
-        for (int64_t s = 0; s < groups; s += 65535)
-            TIGRE_TRY(launch_forward_columns<TP>(g, quads, proj, (int)a0, table + 4 * s,
-                                                 std::min<int64_t>(65535, groups - s), batch,
-                                                 vol_stride, proj_stride, st));
-        return TIGRE_OK;
+    const ColGroups all = column_groups(g, a0, na);
+    const int64_t per = all.four ? 4 : 1;  // angles per group
+    for (int64_t s = 0; s < all.count; s += 65535) {
+        const int64_t cnt = std::min<int64_t>(65535, all.count - s);
+        // without a table the later launches start at their own first angle
+        const int64_t skip = all.table ? 0 : s * per;
+        TIGRE_TRY(launch_forward_columns<TP>(
+            g, quads, proj + skip * n_pix(g), (int)(a0 + skip), na - skip,
+            ColGroups{all.four, all.table ? all.table + 4 * s : nullptr, cnt}, batch, vol_stride,
+            proj_stride, st));
     }
-    return launch_forward_columns<TP>(g, quads, proj, (int)a0, nullptr, na, batch, vol_stride,
-                                      proj_stride, st);
+    return TIGRE_OK;
 }
 
 tigre_status forward_workspace(tigre_geometry* g, tigre_dtype vt, int64_t a0, int64_t na,
@@ -968,11 +995,13 @@ tigre_status forward_workspace(tigre_geometry* g, tigre_dtype vt, int64_t a0, in
     }
     const bool use_quad = !siddon && (g->fwd_path == 0 || g->fwd_path >= 3);
     if (takes_columns(g, a0, na)) {
-        const bool all = a0 == 0 && na == (int64_t)g->angles.size();
-        if (!all && na >= kColsGroupAngles) {
+        if (columns_want_table(g, a0, na)) {
+            cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+            TIGRE_CUDA(cudaStreamIsCapturing(st, &capturing));
             const int* table = nullptr;
             int64_t groups = 0;
-            TIGRE_TRY(range_group_table(g, 1, a0, na, &table, &groups));
+            if (capturing == cudaStreamCaptureStatusNone)
+                TIGRE_TRY(range_group_table(g, 1, a0, na, &table, &groups));
         }
         return g->vol_qxy.ensure(padded_elems(d) * sizeof(float4));  // one set of quads
     }

@@ -105,6 +105,7 @@ struct ColGeom {
     uint32_t SX, SY;  // quads between x and y neighbours
     uint32_t bias;    // of an element index built from split_bits parts
     int ag;  // angles per block: 1 (at four tiles of columns) or kColWarps (at one)
+    int na;     // angles of the launch
     int tiles;  // row tiles of one member
     int64_t vol_stride, proj_stride;  // between a batch's members
 };
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(32 * kColWarps, kColBlocks) fwd_cols_kernel(
         const int q = tile * ROWS + (int)threadIdx.x % ROWS;
         const int g = (int)blockIdx.y * w.ag + (w.ag == 1 ? 0 : warp);
         const int a = order ? order[g] : g;
-        if (a < 0 || pw >= c.nu) return;  // the whole warp
+        if (a < 0 || a >= w.na || pw >= c.nu) return;  // the whole warp
         const FwdAngle* P = params + a_first + a;
         const int layout = P->layout;
         bool active[2];
@@ -283,7 +284,7 @@ tigre_status build_quad_columns(const tigre_geometry_desc& d, const T* vol, floa
 
 template <typename TP>
 tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* proj, int a_first,
-                                    const int* table, int64_t groups, int batch,
+                                    int64_t na, const ColGroups& groups, int batch,
                                     int64_t vol_stride, int64_t proj_stride, cudaStream_t st)
 {
     const FwdConst c = make_fwd_const(g);
@@ -297,21 +298,22 @@ tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* 
     // (512^3 x 360: 94.5 / 93.3, 128^3 x 90: 0.519 / 0.495).
     const bool large = (int64_t)c.nx * c.ny >= 640 * 640;
     const int rows = large && (c.nv >= 224 || c.nv <= 16) ? 16 : 8;
-    const int ag = table ? kColWarps : 1;
+    const int ag = groups.four ? kColWarps : 1;
     const int cols = 2 * (32 / rows) * (kColWarps / ag), tiles = (c.nv + rows - 1) / rows;
-    dim3 grid((unsigned)((c.nu + cols - 1) / cols), (unsigned)groups, (unsigned)(tiles * batch));
+    dim3 grid((unsigned)((c.nu + cols - 1) / cols), (unsigned)groups.count, (unsigned)(tiles * batch));
     ColGeom w;
     w.SX = (uint32_t)(c.nz + 2 * kPad);
     w.SY = w.SX * (uint32_t)(c.nx + 2 * kPad);
     w.bias = 0x4B000000u * (w.SY + w.SX + 1u);
     w.ag = ag;
+    w.na = (int)na;
     w.tiles = tiles;
     w.vol_stride = vol_stride;
     w.proj_stride = proj_stride;
     auto kern = batch > 1 ? (rows == 16 ? fwd_cols_kernel<TP, true, 16> : fwd_cols_kernel<TP, true, 8>)
                           : (rows == 16 ? fwd_cols_kernel<TP, false, 16> : fwd_cols_kernel<TP, false, 8>);
     kern<<<grid, dim3(32, kColWarps), 0, st>>>(quads, proj, (const FwdAngle*)g->fwd_params.ptr, c,
-                                               a_first, table, w);
+                                               a_first, groups.table, w);
     TIGRE_LAUNCHED("fwd_cols_kernel");
     return TIGRE_OK;
 }
@@ -320,8 +322,8 @@ tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* 
     template tigre_status build_quad_columns<T>(const tigre_geometry_desc&, const T*, float4*,  \
                                                 cudaStream_t);                                  \
     template tigre_status launch_forward_columns<T>(tigre_geometry*, const float4*, T*, int,    \
-                                                    const int*, int64_t, int, int64_t, int64_t, \
-                                                    cudaStream_t);
+                                                    int64_t, const ColGroups&, int, int64_t,    \
+                                                    int64_t, cudaStream_t);
 TIGRE_COLS(float)
 TIGRE_COLS(__nv_bfloat16)
 TIGRE_COLS(__half)

@@ -10,13 +10,19 @@ namespace tigre {
 template <typename T>
 tigre_status build_quad_columns(const tigre_geometry_desc& d, const T* vol, float4* out,
                                 cudaStream_t st);
-// Projection of `groups` groups of four angles: table[4 i + j] is an angle
-// relative to a_first or -1; or with a null table of the `groups` angles from
-// a_first, one per block.  A batch's members lie vol_stride quads and
-// proj_stride elements apart.
+// The angles of a launch's blocks: with `four`, block row i projects the angles
+// table[4 i .. 4 i + 3] (relative to the launch's first one, -1 for none), or
+// with a null table 4 i .. 4 i + 3 themselves; otherwise angle i alone.
+struct ColGroups {
+    bool four;
+    const int* table;
+    int64_t count;
+};
+// Projection of the angles [a_first, a_first + na).  A batch's members lie
+// vol_stride quads and proj_stride elements apart.
 template <typename TP>
 tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* proj, int a_first,
-                                    const int* table, int64_t groups, int batch,
+                                    int64_t na, const ColGroups& groups, int batch,
                                     int64_t vol_stride, int64_t proj_stride, cudaStream_t st);
 
 // Exact transpose of the projection of the angles [a0, a0 + na) (adjoint_cols.cu)
