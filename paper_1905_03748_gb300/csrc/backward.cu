@@ -112,8 +112,14 @@ template <typename TP> struct ProjTaps<TP, true> {
 // 16/4 9.13, 8/4 9.36.  Fewer voxels per thread where the columns alone do not
 // fill the chip (blocks at 16 voxels): 192^3 (1728 blocks) OS-SART sweep 8/4
 // 1.51, 16/3 1.63; 128^3 (512) 8/4 0.182, 16/4 0.188, 4/4 0.214; 64^3 (64) 4/4
-// 0.049, 8/4 0.073, 16/4 0.135.  The line between 8 and 16 lies between the 1728
-// blocks of 192^3 and the 4096 of 256^3 (16/4 4.40, 8/4 4.82).
+// 0.049, 8/4 0.073, 16/4 0.135.  The line between 8 and 16: 90 angles, matched 8 /
+// 16, 192^3 (1728 blocks) 0.457 / 0.447, 208^3 (2366) 0.595 / 0.571, 216^3 (2646)
+// 0.666 / 0.698, 256^3 (4096) 1.074 / 1.027; FDK 0.422 / 0.431, 0.547 / 0.554, 0.621 /
+// 0.684, 0.980 / 1.001; SART within 1 %.  From 300 blocks to three per SM (456)
+// again 16: eight voxels make 600 to 912 blocks of at most 608 at a time, the rest
+// a second turn of few (180 angles, 112^3, 392 blocks: matched 4 / 8 / 16 0.277 / 0.293
+// / 0.240, FDK 0.206 / 0.268 / 0.226, SART sweep 1.28 / 1.30 / 1.28; 116^3, 480 blocks
+// 0.289 / 0.298 / 0.304, 0.272 / 0.266 / 0.294, 1.36 / 1.39 / 1.43).
 // Plain (out-of-core, fewer than four angles) buffers: 16 voxels, 5 or 3 blocks.
 constexpr int kBpLaneX = 4;
 template <bool SART, bool QUADP>
@@ -121,7 +127,8 @@ constexpr int bp_blocks_per_sm(int nz)
 {
     return !QUADP ? (SART ? 3 : 5) : SART && nz == 16 ? 3 : 4;
 }
-constexpr int64_t kBpBlocks16 = 2500, kBpBlocks8 = 300;  // blocks at 16 voxels per thread
+// blocks at 16 voxels per thread
+constexpr int64_t kBpBlocks16 = 2500, kBpBlocks8 = 300, kBpBlocksTurn = 3 * 152;
 
 // Members of a batched launch: blockIdx.z = member * chunks + z chunk; member
 // i reads projections proj_stride elements and writes the volume vol_stride
@@ -578,7 +585,7 @@ static tigre_status run_voxel_bp(tigre_geometry* g, const BpConst& c, const TP* 
         if constexpr (QUADP) {
             if (blocks16 < kBpBlocks8)
                 return launch_nz(mode, sart_tag, std::integral_constant<int, 4>{});
-            if (blocks16 < kBpBlocks16)
+            if (blocks16 > kBpBlocksTurn && blocks16 < kBpBlocks16)
                 return launch_nz(mode, sart_tag, std::integral_constant<int, 8>{});
         }
         return launch_nz(mode, sart_tag, std::integral_constant<int, 16>{});
