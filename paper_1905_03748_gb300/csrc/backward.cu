@@ -546,7 +546,6 @@ static tigre_status run_voxel_bp(tigre_geometry* g, const BpConst& c, const TP* 
     const BpAngle* params = (const BpAngle*)g->bp_params.ptr;
     const dim3 block(32, 8);
     ProfScope prof(kProfBackproject, st);
-    // One kernel instance: MODE and SART fixed, NZ voxels per thread.
     // Voxels per thread from one member's blocks, so that a problem's numbers
     // are the same alone and in a batch.
     const int64_t cols = (int64_t)((c.nx + 31) / 32) * ((c.ny + 7) / 8);
@@ -558,27 +557,32 @@ static tigre_status run_voxel_bp(tigre_geometry* g, const BpConst& c, const TP* 
         constexpr int NZ = decltype(nz)::value;
         static_assert(NZ <= kBpNZ, "the row-band bounds assume chunks of at most kBpNZ planes");
         const int chunks = (c.z_end - c.z_first + NZ - 1) / NZ;
-        dim3 grid((unsigned)((c.nx + 31) / 32), (unsigned)((c.ny + 7) / 8),
-                  (unsigned)((int64_t)chunks * batch));
-        if (grid.y > 65535 || (int64_t)chunks * batch > 65535)
+        dim3 grid((unsigned)((c.nx + 31) / 32), (unsigned)((c.ny + 7) / 8), (unsigned)chunks);
+        if (grid.y > 65535 || chunks > 65535 ||
+            (int64_t)((c.z_end - c.z_first + kBpNZ - 1) / kBpNZ) * batch > 65535)
             return fail(TIGRE_ERR_UNSUPPORTED, "volume too large");
-        BpBatch bt;
-        if (batch > 1) {
-            bt.chunks = chunks;
-            bt.proj_stride = (int64_t)pelems;
-            bt.vol_stride = (int64_t)c.nx * c.ny * c.nz;
-        }
         // (single launches take the instance without member offsets: FDK at
         // 512^3 x 360 33.3 ms against 37.8 with them)
         if constexpr (QUADP && !S) {
             if (batch > 1) {
-                bp_voxel_kernel<TP, TV, NZ, M, S, QUADP, true><<<grid, block, 0, st>>>(
-                    pp, vol, params, c, (int)a0, (int)na, accumulate, lambda, nonneg, bt);
+                BpBatch bt;
+                bt.chunks = chunks;
+                bt.proj_stride = (int64_t)pelems;
+                bt.vol_stride = (int64_t)c.nx * c.ny * c.nz;
+                // small chunks of many deep members may exceed a grid's z
+                // extent: as many members at a time as fit
+                for (int i = 0; i < batch; i += 65535 / chunks) {
+                    if (i > 0) TIGRE_LAUNCHED("bp_voxel_kernel");
+                    grid.z = (unsigned)(std::min(batch - i, 65535 / chunks) * chunks);
+                    bp_voxel_kernel<TP, TV, NZ, M, S, QUADP, true><<<grid, block, 0, st>>>(
+                        pp + i * bt.proj_stride, vol + i * bt.vol_stride, params, c, (int)a0,
+                        (int)na, accumulate, lambda, nonneg, bt);
+                }
                 return TIGRE_OK;
             }
         }
         bp_voxel_kernel<TP, TV, NZ, M, S, QUADP><<<grid, block, 0, st>>>(
-            pp, vol, params, c, (int)a0, (int)na, S ? 0 : accumulate, lambda, nonneg, bt);
+            pp, vol, params, c, (int)a0, (int)na, S ? 0 : accumulate, lambda, nonneg, BpBatch{});
         return TIGRE_OK;
     };
     auto launch = [&](auto mode, auto sart_tag) -> tigre_status {
