@@ -503,7 +503,8 @@ tigre_status backward_workspace(tigre_geometry* g, tigre_dtype pt, tigre_bp_weig
     const tigre_geometry_desc& d = g->desc;
     if (w == TIGRE_BP_EXACT_ADJOINT) {
         if (padded_elems(d) >= (size_t)INT32_MAX) return TIGRE_OK;  // refused by the operator
-        if (adjoint_takes_columns(g, na)) return g->adj_xy.ensure(padded_elems(d) * sizeof(float4));
+        if (adjoint_takes_columns(g, na))
+            return g->adj_quads.ensure(padded_elems(d) * sizeof(float4));
         bool need[2] = {false, false};
         for (int64_t a = a0; a < a0 + na; ++a) need[g->layout[(size_t)a]] = true;
         DeviceBuffer* bufs[2] = {&g->adj_xy, &g->adj_yx};
@@ -725,11 +726,10 @@ static tigre_status launch_adjoint(tigre_geometry* g, const TP* proj, TV* vol, i
     const FwdConst c = make_fwd_const(g);
     if (adjoint_takes_columns(g, na)) {
         const size_t quads = padded_elems(d) * sizeof(float4);
-        TIGRE_TRY(g->adj_xy.ensure(quads));
-        g->adj_xy.tag = 0;
-        TIGRE_CUDA(cudaMemsetAsync(g->adj_xy.ptr, 0, quads, st));
+        TIGRE_TRY(g->adj_quads.ensure(quads));
+        TIGRE_CUDA(cudaMemsetAsync(g->adj_quads.ptr, 0, quads, st));
         ProfScope prof(kProfAdjoint, st);
-        return launch_adjoint_columns<TP, TV>(g, proj, (float4*)g->adj_xy.ptr, vol, a0, na,
+        return launch_adjoint_columns<TP, TV>(g, proj, (float4*)g->adj_quads.ptr, vol, a0, na,
                                               accumulate, st);
     }
     bool need[2] = {false, false};

@@ -191,9 +191,11 @@ struct tigre_geometry {
                                       // projector keeps its one set in vol_qxy)
     tigre::DeviceBuffer vol_qyx;
     tigre::DeviceBuffer proj_pad;     // zero-bordered projections for the backprojector
-    tigre::DeviceBuffer adj_xy;       // FP32 padded accumulators of the exact adjoint (the
-                                      // column scatter keeps its quads in adj_xy)
+    // Accumulators of the exact adjoint.  The two scatters have their own, so
+    // that neither is reallocated under a captured graph of the other's calls.
+    tigre::DeviceBuffer adj_xy;       // FP32 padded volumes of the scalar scatter
     tigre::DeviceBuffer adj_yx;
+    tigre::DeviceBuffer adj_quads;    // quads of the column scatter
     tigre::DeviceBuffer scratch_vol;  // FP32 volume-sized scratch
     tigre::DeviceBuffer scratch_red;  // reduction partials / device scalars
     std::vector<int> layout;          // forward-projector layout per angle (host copy)

@@ -118,7 +118,8 @@ std::vector<uint64_t> workspace_signature(const tigre_geometry* g)
 {
     std::vector<uint64_t> sig;
     for (const DeviceBuffer* b : {&g->vol_xy, &g->vol_yx, &g->vol_qxy, &g->vol_qyx, &g->proj_pad,
-                                  &g->adj_xy, &g->adj_yx, &g->err_flag, &g->brick_prange}) {
+                                  &g->adj_xy, &g->adj_yx, &g->adj_quads, &g->err_flag,
+                                  &g->brick_prange}) {
         sig.push_back((uint64_t)(uintptr_t)b->ptr);
         sig.push_back(b->tag);
     }
@@ -401,6 +402,7 @@ tigre_status tigre_geometry_destroy(tigre_geometry_t g)
     g->proj_pad.release();
     g->adj_xy.release();
     g->adj_yx.release();
+    g->adj_quads.release();
     g->err_flag.release();
     g->brick_prange.release();
     g->scratch_vol.release();
