@@ -494,6 +494,25 @@ static bool adjoint_takes_columns(const tigre_geometry* g, int64_t na)
     return g->projector == TIGRE_PROJ_INTERPOLATED && column_warps_pay(g, na);
 }
 
+// The column scatter's accumulators (16 bytes per padded voxel; the scalar
+// scatter's are 4 per layout in use).  *have = false where the memory does not
+// suffice, or where they are missing inside a stream's capture, which may not
+// allocate: the scalar scatter then takes the call.  (No stream: not capturing.)
+static tigre_status adjoint_quads(tigre_geometry* g, const cudaStream_t* st, bool* have)
+{
+    const size_t bytes = padded_elems(g->desc) * sizeof(float4);
+    *have = g->adj_quads.ptr != nullptr;
+    if (*have) return TIGRE_OK;
+    if (st) {
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        TIGRE_CUDA(cudaStreamIsCapturing(*st, &capturing));
+        if (capturing != cudaStreamCaptureStatusNone) return TIGRE_OK;
+    }
+    const tigre_status s = g->adj_quads.ensure(bytes);
+    *have = s == TIGRE_OK;
+    return s == TIGRE_ERR_OOM ? TIGRE_OK : s;
+}
+
 tigre_status backward_workspace(tigre_geometry* g, tigre_dtype pt, tigre_bp_weight w, int64_t a0,
                                 int64_t na)
 {
@@ -503,8 +522,11 @@ tigre_status backward_workspace(tigre_geometry* g, tigre_dtype pt, tigre_bp_weig
     const tigre_geometry_desc& d = g->desc;
     if (w == TIGRE_BP_EXACT_ADJOINT) {
         if (padded_elems(d) >= (size_t)INT32_MAX) return TIGRE_OK;  // refused by the operator
-        if (adjoint_takes_columns(g, na))
-            return g->adj_quads.ensure(padded_elems(d) * sizeof(float4));
+        if (adjoint_takes_columns(g, na)) {
+            bool have = false;
+            TIGRE_TRY(adjoint_quads(g, nullptr, &have));
+            if (have) return TIGRE_OK;
+        }
         bool need[2] = {false, false};
         for (int64_t a = a0; a < a0 + na; ++a) need[g->layout[(size_t)a]] = true;
         DeviceBuffer* bufs[2] = {&g->adj_xy, &g->adj_yx};
@@ -724,10 +746,10 @@ static tigre_status launch_adjoint(tigre_geometry* g, const TP* proj, TV* vol, i
     if (padded_elems(d) >= (size_t)INT32_MAX)
         return fail(TIGRE_ERR_UNSUPPORTED, "exact adjoint needs (nx+4)(ny+4)(nz+4) < 2^31");
     const FwdConst c = make_fwd_const(g);
-    if (adjoint_takes_columns(g, na)) {
-        const size_t quads = padded_elems(d) * sizeof(float4);
-        TIGRE_TRY(g->adj_quads.ensure(quads));
-        TIGRE_CUDA(cudaMemsetAsync(g->adj_quads.ptr, 0, quads, st));
+    bool columns = adjoint_takes_columns(g, na);
+    if (columns) TIGRE_TRY(adjoint_quads(g, &st, &columns));
+    if (columns) {
+        TIGRE_CUDA(cudaMemsetAsync(g->adj_quads.ptr, 0, padded_elems(d) * sizeof(float4), st));
         ProfScope prof(kProfAdjoint, st);
         return launch_adjoint_columns<TP, TV>(g, proj, (float4*)g->adj_quads.ptr, vol, a0, na,
                                               accumulate, st);
