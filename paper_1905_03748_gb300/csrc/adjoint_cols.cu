@@ -111,14 +111,14 @@ __global__ void __launch_bounds__(32 * kAdjWarps) adj_cols_kernel(
     }
 }
 
-// vol[z][y][x] (+)= what the four cells around it gave its corner of plane z.
+// vol[z][y][x] = what the four cells around it gave its corner of plane z.
 // A block takes 32 planes x 32 x and marches `rows` y rows: a lane is a plane,
 // a thread four neighbouring x, whose sums from the row of cells below stay in
 // registers; each row is transposed in shared memory and written along x.
 template <typename TV>
 __global__ void __launch_bounds__(256) adj_cols_finish_kernel(const float4* __restrict__ acc,
                                                               TV* __restrict__ vol, int nx, int ny,
-                                                              int nz, int rows, int accumulate)
+                                                              int nz, int rows)
 {
     __shared__ float tile[32][33];  // [z][x]
     const int PX = nx + 2 * kPad, PS = nz + 2 * kPad;
@@ -142,11 +142,8 @@ __global__ void __launch_bounds__(256) adj_cols_finish_kernel(const float4* __re
             __syncthreads();
             const int x = x0 + (int)threadIdx.x;
             for (int k = threadIdx.y; k < 32 && z0 + k < nz; k += 8)
-                if (x < nx) {
-                    TV* o = vol + ((int64_t)(z0 + k) * ny + y) * nx + x;
-                    const float v = tile[k][threadIdx.x];
-                    *o = from_f32<TV>(accumulate ? to_f32<TV>(*o) + v : v);
-                }
+                if (x < nx)
+                    vol[((int64_t)(z0 + k) * ny + y) * nx + x] = from_f32<TV>(tile[k][threadIdx.x]);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) below[i] = e[i + 1].z + e[i].w;
@@ -157,7 +154,7 @@ __global__ void __launch_bounds__(256) adj_cols_finish_kernel(const float4* __re
 
 template <typename TP, typename TV>
 tigre_status launch_adjoint_columns(tigre_geometry* g, const TP* proj, float4* acc, TV* vol,
-                                    int64_t a0, int64_t na, int accumulate, cudaStream_t st)
+                                    int64_t a0, int64_t na, cudaStream_t st)
 {
     const FwdConst c = make_fwd_const(g);
     const uint32_t SX = (uint32_t)(c.nz + 2 * kPad), SY = SX * (uint32_t)(c.nx + 2 * kPad);
@@ -174,15 +171,14 @@ tigre_status launch_adjoint_columns(tigre_geometry* g, const TP* proj, float4* a
     const int rows = std::max(16, (c.ny + 65534) / 65535);
     dim3 grid((unsigned)((c.nz + 31) / 32), (unsigned)((c.nx + 31) / 32),
               (unsigned)((c.ny + rows - 1) / rows));
-    adj_cols_finish_kernel<TV><<<grid, dim3(32, 8), 0, st>>>(acc, vol, c.nx, c.ny, c.nz, rows,
-                                                             accumulate);
+    adj_cols_finish_kernel<TV><<<grid, dim3(32, 8), 0, st>>>(acc, vol, c.nx, c.ny, c.nz, rows);
     TIGRE_LAUNCHED("adj_cols_finish_kernel");
     return TIGRE_OK;
 }
 
 #define TIGRE_ADJ(TP, TV)                                                                        \
     template tigre_status launch_adjoint_columns<TP, TV>(tigre_geometry*, const TP*, float4*,    \
-                                                         TV*, int64_t, int64_t, int, cudaStream_t);
+                                                         TV*, int64_t, int64_t, cudaStream_t);
 #define TIGRE_ADJ_ALL(TP)          \
     TIGRE_ADJ(TP, float)           \
     TIGRE_ADJ(TP, __nv_bfloat16)   \

@@ -746,13 +746,12 @@ static tigre_status launch_adjoint(tigre_geometry* g, const TP* proj, TV* vol, i
     if (padded_elems(d) >= (size_t)INT32_MAX)
         return fail(TIGRE_ERR_UNSUPPORTED, "exact adjoint needs (nx+4)(ny+4)(nz+4) < 2^31");
     const FwdConst c = make_fwd_const(g);
-    bool columns = adjoint_takes_columns(g, na);
+    bool columns = !accumulate && adjoint_takes_columns(g, na);  // (it overwrites the volume)
     if (columns) TIGRE_TRY(adjoint_quads(g, &st, &columns));
     if (columns) {
         TIGRE_CUDA(cudaMemsetAsync(g->adj_quads.ptr, 0, padded_elems(d) * sizeof(float4), st));
         ProfScope prof(kProfAdjoint, st);
-        return launch_adjoint_columns<TP, TV>(g, proj, (float4*)g->adj_quads.ptr, vol, a0, na,
-                                              accumulate, st);
+        return launch_adjoint_columns<TP, TV>(g, proj, (float4*)g->adj_quads.ptr, vol, a0, na, st);
     }
     bool need[2] = {false, false};
     for (int64_t a = a0; a < a0 + na; ++a) need[g->layout[(size_t)a]] = true;

@@ -29,7 +29,7 @@ tigre_status launch_forward_columns(tigre_geometry* g, const float4* quads, TP* 
 // through padded_elems accumulator quads, zeroed by the caller.
 template <typename TP, typename TV>
 tigre_status launch_adjoint_columns(tigre_geometry* g, const TP* proj, float4* acc, TV* vol,
-                                    int64_t a0, int64_t na, int accumulate, cudaStream_t st);
+                                    int64_t a0, int64_t na, cudaStream_t st);
 
 // Whether warps of detector rows suit a call of na angles (forward.cu).
 bool column_warps_pay(const tigre_geometry* g, int64_t na);
