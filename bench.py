@@ -318,8 +318,11 @@ def run_ours(args):
            "roofline": {"kernel": "fwd_cols_kernel", "bound": "l1", "achieved": l1_achieved,
                         "peak": l1_peak, "unit": "TB/s", "frac": l1_achieved / l1_peak,
                         "traffic": traffic,
-                        "per_unit": f"{L1_BYTES_PER_SAMPLE} B gathered per quadrature sample "
-                                    f"(eight FP32 taps) x {samples} samples per launch",
+                        "per_unit": f"{L1_BYTES_PER_SAMPLE} B per quadrature sample (eight FP32 "
+                                    f"taps) x {samples} samples per launch: algorithmic bytes, "
+                                    "those served from registers while a ray stays in a cell "
+                                    "included, so frac is no utilisation and 1 is no bound; the "
+                                    "measured one is ncu_sol.l1tex_data_pipe_lsu_wavefronts_pct",
                         "peak_source": f"{n_sm} SMs (device query) x 128 B per clock (L1 data "
                                        f"path) x max SM clock {sm_max_mhz:.0f} MHz (derived; "
                                        "no measured L1 peak exists)",
