@@ -43,6 +43,19 @@ def test_rows_equal_the_quad_kernel(tigre, name):
     assert torch.equal(out[tigre.FWD_QUAD], out[tigre.FWD_AUTO])
 
 
+def test_more_than_2_28_quads(tigre):
+    """Byte offsets beyond 32 bits (704 x 696 x 646 padded voxels), ragged tiles."""
+    geo, ang = geometry((700, 692, 642), 203, 349), synth.angles(11, first=0.3)
+    with tigre.Geometry(geo, ang) as G:
+        v = torch.rand(tuple(G.vol_shape), device="cuda",
+                       generator=torch.Generator(device="cuda").manual_seed(5))
+        n0 = tigre.tigre_launch_count()
+        out = G.forward(v)
+        assert tigre.tigre_launch_count() - n0 == 2  # columns
+        tigre.tigre_geometry_set_forward_path(G.handle, tigre.FWD_QUAD)
+        assert torch.isfinite(out).all() and torch.equal(out, G.forward(v))
+
+
 @pytest.mark.parametrize("graph", [False, True])
 def test_batched_16_row_warps(tigre, graph):
     """Members of a batch (two iterations of CGLS) equal their problems alone."""
