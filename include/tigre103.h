@@ -424,16 +424,18 @@ TIGRE_API tigre_status tigre_geometry_set_projector(tigre_geometry_t geo, int pr
  * each z-slab (0 = default 512).  Rays resident on the GPU at one time then
  * read one brick's planes, which stay in L2; at 3072^2 a single quad plane
  * of the slab is larger than L2.  In-core projections on the automatic path
- * (F32 volume and projections) that take the quad gather kernel march the
- * same bricks when the volume is wider than one brick; the column kernel has
- * no bricks.  Only the partial sums' order changes. */
+ * (F32 volume and projections) march the same bricks when the volume is wider
+ * than one brick and the projection of all the handle's angles takes the quad
+ * gather kernel; the column kernel has no bricks, and ranges of angles follow
+ * the full range.  Only the partial sums' order changes. */
 TIGRE_API tigre_status tigre_geometry_set_brick(tigre_geometry_t geo, int64_t edge);
 
 /* Kernel choice for this handle's Sec. 2.1 projector (no counterpart in the
  * paper): 0 = automatic (the column
  * kernel, whose warps are detector rows and which reads one set of quads with
- * z fastest, for calls of at least three angles and 250,000 rays on detectors
- * of at least 16 rows that lie at most 1.9 planes apart at the axis; otherwise
+ * z fastest, for calls of at least three angles and 250,000 rays, 120,000 of
+ * which cross the volume, on detectors of at least 16 rows that lie at most 1.9
+ * planes apart at the axis, with more rows or angles on wide volumes; otherwise
  * the quad gather kernel, with 2 angles per warp when the rays of one pixel at
  * paired angles stay within 16 voxels of each other), 1 = scalar
  * L1 gather kernel, 2 = shared-memory slab kernel (TMA-staged; only for

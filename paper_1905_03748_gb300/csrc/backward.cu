@@ -19,17 +19,21 @@
 // element (r, c) holds the four FP32 bilinear coefficients of the cell
 // (c, c+1) x (r, r+1) for every storage type, so a voxel-angle pair costs one
 // aligned 16-byte load and three FMAs instead of four scalar loads, their
-// addresses and three lerps (the kernel is bound by instruction issue).  Out-of-core slab launches read a
-// band of rows per slab, which spans the cone's spread (hundreds of rows at
-// 3072^3): they build quads of a quarter of the angles at a time, in the
-// bytes a plain band of all angles takes.
+// addresses and three lerps; the L1 data pipe that serves those loads is then
+// the bound.  Out-of-core slab launches read a band of rows per slab, which
+// spans the cone's spread (hundreds of rows at 3072^3): they build quads of a
+// quarter of the angles at a time, in the bytes a plain band of all angles
+// takes.
 // Grid order: x-tiles fastest, z-chunks slowest, so resident blocks share one
 // band of detector rows per angle in L2.
 //
-// Exact adjoint: the transpose of the forward projector, each ray scattering
-// h * trilinear weight * y into the 8 corner voxels of each of its samples
-// (FP32 atomics into padded accumulators in the same two layouts as the
-// forward projector, so a warp's atomics hit adjacent addresses).
+// Exact adjoint: the transpose of the forward projector.  Calls of many rays
+// take the column scatter (adjoint_cols.cu: quad accumulators, two vector
+// reductions per cell a ray crosses).  For few rays, the Siddon projector and
+// where the quads do not fit, each ray scatters h * trilinear weight * y into
+// the 8 corner voxels of each of its samples here (FP32 atomics into padded
+// accumulators in the row-warp projector's two layouts, so a warp's atomics
+// hit adjacent addresses).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -200,7 +204,9 @@ __global__ void __launch_bounds__(256, (bp_blocks_per_sm<SART, QUADP>(NZ))) bp_v
         const float pv0 = fmaf(Zb * mag, c.inv_dv, pv_off);
         const float dpv = c.dz * mag * c.inv_dv;
         float tu = 0.0f;  // bilinear weight of the all-ones image along u
-        bool inner = true;  // and along v: 1 where every cell lies on the detector
+        // and along v: exactly 1 where every cell lies on the detector, where
+        // (1 - fv) + fv would round (x is as near 64 bits as with it)
+        bool inner = true;
         if (SART) {
             tu = ((unsigned)(ip - kPad) < (unsigned)c.nu ? 1.0f - fu : 0.0f) +
                  ((unsigned)(ip - kPad + 1) < (unsigned)c.nu ? fu : 0.0f);
@@ -487,8 +493,13 @@ static bool bp_quads_addressable(const BpConst& c)
     return (int64_t)c.PU * c.PV < ((int64_t)1 << 28);
 }
 
-// Whether an exact adjoint takes the column scatter (adjoint_cols.cu), by the
-// forward projector's rule.
+// Whether an exact adjoint takes the column scatter (adjoint_cols.cu): by the
+// lines drawn for the forward projector, which also bound its workspace (16
+// bytes per padded voxel) to calls of many rays.  The scatter itself was the
+// faster one wherever it was tried, its memset and read of every voxel's 16
+// bytes included (column / scalar ms): 1024^3, 3 angles under 160 x 600 10.1 /
+// 25.4, under 1024^2 39.5 / 70.0; 512^3, 3 angles under 512^2 4.8 / 10.1; 128^3
+// under 128^2, 8 angles 0.15 / 1.09; 64^3 under 128^2, 2 angles 0.053 / 0.069.
 static bool adjoint_takes_columns(const tigre_geometry* g, int64_t na)
 {
     return g->projector == TIGRE_PROJ_INTERPOLATED && column_warps_pay(g, na);

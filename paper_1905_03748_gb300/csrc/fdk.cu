@@ -209,7 +209,12 @@ tigre_status fdk_impl(tigre_geometry* g, const void* proj, tigre_dtype pt, void*
         status = dispatch_dtype(pt, [&](auto tag) -> tigre_status {
             using TP = decltype(tag);
             // Blocks of 8 rows up to 2048 columns (73 KB: three per SM), of 4
-            // up to 8192 (164 KB); longer rows one by one.  An instance's
+            // up to 8192 (164 KB: one per SM); longer rows one by one.  360
+            // angles, whole call, ms with 8 / 4 / 2 / 1 rows a block and the
+            // row-by-row kernel: 512 columns x 64 rows 0.77 / 0.77 / 0.78 / 0.82 /
+            // 2.05, 2048 x 64 3.16 / 3.23 / 3.52 / 3.92 / 17.2, 2048 x 9 1.20 / 1.02 /
+            // 0.97 / 0.95 / 3.25; 4096 x 9 - / 2.96 / 2.52 / 2.38 / 10.3, 8192 x 9 - /
+            // 13.2 / 11.9 / 9.0 / 38.4, 8192 x 1 - / 5.0 / 4.2 / 1.6 / 6.2.  An instance's
             // shared-memory limit is the process's: a call beyond the default
             // 48 KB sets it to what the instance's longest rows need, never to
             // its own rows' bytes, which another thread's launch may exceed

@@ -9,8 +9,8 @@
 //
 // Whole volumes are projected by the column kernel (forward_cols.cu) where its
 // rule allows (takes_columns); this file holds that choice and the other
-// kernels: few rays, few or widely spaced detector rows, slabs of a volume, and
-// the paths a caller selects.
+// kernels: few crossing rays, few or widely spaced detector rows, slabs of a
+// volume, and the paths a caller selects.
 //
 // GB300 design of the row-warp kernels:
 //  * The volume is copied once per call into two zero-padded layouts (x
