@@ -105,7 +105,7 @@ struct ColGeom {
     uint32_t SX, SY;  // quads between x and y neighbours
     uint32_t bias;    // of an element index built from split_bits parts
     int ag;  // angles per block: 1 (at four tiles of columns) or kColWarps (at one)
-    int na;     // angles of the launch
+    int na;     // angles of the launch (a batch has its table, or one angle a block)
     int tiles;  // row tiles of one member
     int64_t vol_stride, proj_stride;  // between a batch's members
 };
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(32 * kColWarps, kColBlocks) fwd_cols_kernel(
         const int q = tile * ROWS + (int)threadIdx.x % ROWS;
         const int g = (int)blockIdx.y * w.ag + (w.ag == 1 ? 0 : warp);
         const int a = order ? order[g] : g;
-        if (a < 0 || a >= w.na || pw >= c.nu) return;  // the whole warp
+        if (a < 0 || (!BATCH && a >= w.na) || pw >= c.nu) return;  // the whole warp
         const FwdAngle* P = params + a_first + a;
         const int layout = P->layout;
         bool active[2];
