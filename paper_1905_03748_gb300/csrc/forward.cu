@@ -975,9 +975,43 @@ static tigre_status run_columns(tigre_geometry* g, const float4* quads, TP* proj
     return TIGRE_OK;
 }
 
-tigre_status forward_workspace(tigre_geometry* g, tigre_dtype vt, int64_t a0, int64_t na,
-                               cudaStream_t st)
+// Whether this call takes the column projector: by the rule, and also where
+// the quad kernel would be the faster one but a second set of quads does not
+// fit beside the first, or is missing, as may be its table of angle pairs,
+// inside a stream capture, which may not allocate (the results are the same
+// bits).
+static tigre_status forward_takes_columns(tigre_geometry* g, tigre_dtype vt, int64_t a0, int64_t na,
+                                          cudaStream_t st, bool* columns)
 {
+    *columns = takes_columns(g, a0, na);
+    if (*columns || g->fwd_path != 0 || g->projector != TIGRE_PROJ_INTERPOLATED ||
+        in_core_bricks(g, vt))
+        return TIGRE_OK;
+    const size_t bytes = padded_elems(g->desc) * sizeof(float4);
+    bool need[2];
+    needed_layouts(g, a0, na, need);
+    const bool second = need[1] && g->vol_qyx.bytes < bytes;
+    const bool pairs = g->auto_angle_group == 2 && na < (int64_t)g->angles.size() &&
+                       g->range_groups[0].find({a0, na}) == g->range_groups[0].end();
+    if (!second && !pairs) return TIGRE_OK;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    TIGRE_CUDA(cudaStreamIsCapturing(st, &capturing));
+    if (capturing != cudaStreamCaptureStatusNone) {
+        *columns = g->vol_qxy.bytes >= bytes;
+        return TIGRE_OK;
+    }
+    if (!second) return TIGRE_OK;
+    if (need[0]) TIGRE_TRY(g->vol_qxy.ensure(bytes));
+    const tigre_status s = g->vol_qyx.ensure(bytes);
+    *columns = s == TIGRE_ERR_OOM && g->vol_qxy.bytes >= bytes;
+    return *columns ? TIGRE_OK : s;
+}
+
+// forward_workspace, and whether the call takes the column projector.
+static tigre_status prepare_forward(tigre_geometry* g, tigre_dtype vt, int64_t a0, int64_t na,
+                                    cudaStream_t st, bool* columns)
+{
+    *columns = false;
     TIGRE_TRY(check_geometry(g));
     TIGRE_TRY(check_range(g, a0, na));
     if (!dtype_ok(vt)) return fail(TIGRE_ERR_INVALID_ARG, "bad dtype");
@@ -994,7 +1028,8 @@ tigre_status forward_workspace(tigre_geometry* g, tigre_dtype vt, int64_t a0, in
         return tma_workspace(g, dtype_size(vt), need);
     }
     const bool use_quad = !siddon && (g->fwd_path == 0 || g->fwd_path >= 3);
-    if (takes_columns(g, a0, na)) {
+    TIGRE_TRY(forward_takes_columns(g, vt, a0, na, st, columns));
+    if (*columns) {
         if (columns_want_table(g, a0, na)) {
             cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
             TIGRE_CUDA(cudaStreamIsCapturing(st, &capturing));
@@ -1023,6 +1058,13 @@ tigre_status forward_workspace(tigre_geometry* g, tigre_dtype vt, int64_t a0, in
     return TIGRE_OK;
 }
 
+tigre_status forward_workspace(tigre_geometry* g, tigre_dtype vt, int64_t a0, int64_t na,
+                               cudaStream_t st)
+{
+    bool columns;
+    return prepare_forward(g, vt, a0, na, st, &columns);
+}
+
 tigre_status forward_impl(tigre_geometry* g, const void* vol, tigre_dtype vt, void* proj,
                           tigre_dtype pt, int64_t a0, int64_t na, cudaStream_t st)
 {
@@ -1037,7 +1079,8 @@ tigre_status forward_impl(tigre_geometry* g, const void* vol, tigre_dtype vt, vo
     if (d.n_det[1] > 65535 * 8)
         return fail(TIGRE_ERR_UNSUPPORTED, "detector too large for one launch");
     const FwdConst c = make_fwd_const(g);
-    TIGRE_TRY(forward_workspace(g, vt, a0, na, st));
+    bool columns;
+    TIGRE_TRY(prepare_forward(g, vt, a0, na, st, &columns));
     bool need[2];
     needed_layouts(g, a0, na, need);
     const bool siddon = g->projector == TIGRE_PROJ_SIDDON;
@@ -1067,7 +1110,7 @@ tigre_status forward_impl(tigre_geometry* g, const void* vol, tigre_dtype vt, vo
         DeviceBuffer* bufs[2] = {&g->vol_xy, &g->vol_yx};
         DeviceBuffer* qbufs[2] = {&g->vol_qxy, &g->vol_qyx};
         static_assert(sizeof(Q) == 4 * sizeof(float), "a quad is four FP32 coefficients");
-        if (takes_columns(g, a0, na)) {
+        if (columns) {
             if (d.n_voxel[2] + 2 * kPad > 65535)
                 return fail(TIGRE_ERR_UNSUPPORTED, "volume too deep for one launch");
             float4* quads = (float4*)g->vol_qxy.ptr;
